@@ -1,5 +1,5 @@
-// Tensor-core (tcgen05) inference of the warm-start network, called by the
-// C ABI in bbp_warm.cu.
+// Tensor-core (tcgen05) inference of the warm-start network and its training
+// step, called by the C ABI in bbp_warm.cu.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -41,6 +41,13 @@ int infer_tc_syndromes_smem(const Geo& g, int M);
 // ordered (syndrome, coset, message), the features computed in the kernel.
 cudaError_t infer_tc_syndromes(const float* theta, const uint8_t* synd, long long B, const Geo& g, int M, double p,
                                float alpha, float* msgs, void* workspace, cudaStream_t st);
+
+// One training step over N rows (bbp_warm_train_step; bbp_warm_train.cu) and
+// its scratch.
+size_t train_workspace_bytes(long long N);
+cudaError_t train_step(float* theta, float* adam_m, float* adam_v, int32_t step, float lr, const float* feats,
+                       const float* targets, const int32_t* lens, long long N, float* grad, float* loss_sum,
+                       void* workspace, cudaStream_t st);
 
 }  // namespace warm
 }  // namespace bbp
