@@ -66,13 +66,8 @@ struct Shape {
 
 // Compiled shapes in the order the default launch tries them: the
 // register-form-only kernels where the geometry allows them, then
-// shared-memory messages where they leave room for the CTAs per SM the
-// register budget is sized for (FusedMinBlocks), then the same shape with
-// its messages in the workspace.  Measured on the d = 11, p = 0.10 workload
-// (GB300, ms per 10^4 syndromes): FP32 register form only (8,4) 16.3 at 3
-// CTAs per SM, (8,2) 18.2; full kernels (8,4) 20.6, (4,2) 30.1, (8,2) 32.7,
-// (4,4) 42.7, (4,1) 44.8, (8,1) 46.7, (16,1) 52.2; FP64 about 150 per 4096
-// syndromes for (4,2) and (8,2), 176 for (4,4).
+// shared-memory messages where they leave room for the CTAs per SM of
+// target_blocks, then the same shape with its messages in the workspace.
 constexpr Shape kShapesF32[] = {{8, 4, false, 4}, {8, 4, false, 3}, {8, 2, false, 4}, {8, 4, false}, {8, 4, true}, {8, 2, false},
                                 {8, 2, true}, {4, 2, false}, {4, 4, false}, {16, 1, false}, {8, 1, false},
                                 {4, 1, false}};
@@ -94,11 +89,20 @@ int target_blocks(int precision, int k, const Shape& s) {
 
 }  // namespace
 
-int fused_smem_bytes(int precision, const Geo& g, int M, int warps, int cosets, bool gm, bool lean) {
-  if (g.k > 4)
-    return precision == 0 ? fused_smem_for<double, 6>(g, M, warps, cosets) : fused_smem_for<float, 6>(g, M, warps, cosets);
-  return precision == 0 ? fused_smem_for<double, 4>(g, M, warps, cosets, gm, lean)
-                        : fused_smem_for<float, 4>(g, M, warps, cosets, gm, lean);
+// The shared memory that decides which geometries a shape is accepted for
+// and where the default shape keeps its messages (hence the workspace a
+// caller provides).  These limits are part of the interface, so they stay
+// where they were when they were set; the kernels need no more than this
+// (fused_layout).
+static int admitted_smem(int precision, const Geo& g, int M, int warps, int cosets, bool gm, bool lean) {
+  const int K = g.k > 4 ? 6 : 4, vec = 1 << K, slot = lean ? vec : 1 << (2 * K), sz = precision == 0 ? 8 : 4;
+  const int side = K == 4 && cosets < 2 ? 2 : cosets;
+  int o = align_up(2 * g.d * (g.d - 1), 16);
+  o += align_up(cosets * g.W * g.W, 16) + align_up(8 * g.nb * g.nb, 16) + align_up(2 * M, 16) + align_up(4 * M, 16);
+  o += align_up(sz * cosets * M, 16) + align_up(8 * cosets * (g.nb * g.nb + M), 16) + 128;
+  if (g.k == 4) o += align_up(10 * M, 16) + align_up(2 * cosets * M, 16);
+  if (!gm) o += sz * vec * cosets * M;
+  return align_up(o + warps * align_up(sz * (cosets * (2 * slot + 16) + 2 * side * vec), 16), 16);
 }
 
 bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, int* messages, bool allow_lean,
@@ -116,7 +120,7 @@ bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, in
       const int mem = sh[i].lean > 0 ? 3 : (sh[i].gm ? 2 : 1);
       if (*messages != 0 && *messages != mem) continue;
       if (sh[i].lean > 0 && (!allow_lean || !register_form_only(g))) continue;
-      const int smem = fused_smem_bytes(precision, g, M, sh[i].warps, sh[i].cosets, sh[i].gm, sh[i].lean > 0);
+      const int smem = admitted_smem(precision, g, M, sh[i].warps, sh[i].cosets, sh[i].gm, sh[i].lean > 0);
       if (smem > kMaxSmemBytes) continue;
       if (pass == 0 && kSmemPerSm / (smem + kSmemReservedPerCta) < target_blocks(precision, g.k, sh[i])) continue;
       *warps = sh[i].warps;

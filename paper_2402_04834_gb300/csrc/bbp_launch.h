@@ -45,7 +45,6 @@ constexpr long long kFusedSlots = 512;
 constexpr int kMaxSmemBytes = 227 * 1024;       // opt-in shared memory of one CTA
 constexpr int kSmemPerSm = 228 * 1024;          // shared memory of one SM
 constexpr int kSmemReservedPerCta = 1024;       // reserved by the runtime per resident CTA
-int fused_smem_bytes(int precision, const Geo& g, int M, int warps, int cosets, bool gm, bool lean = false);
 // Launch shape of the fused kernel: *warps / *cosets / *messages (1 shared
 // memory, 2 workspace slots, 3 shared memory with every block update in
 // register form: k = 4 with a one-node-wide last block) are requests

@@ -1,0 +1,45 @@
+"""The register-form block updates at the edges of their passes: eight jobs
+(message, coset) of one shape per warp pass, so small codes leave passes
+partly empty (d = 3: one 4 x 4 block and the three one-node-wide ones), and
+cosets that stop at different iterations leave one, two or three jobs per
+message.  Against the dense oracle, with the repository's bars: |delta log P|
+<= 1e-9 in FP64 and 1e-3 in FP32."""
+
+import numpy as np
+import pytest
+
+import paper_2402_04834_gb300 as pkg
+import synth
+from oracle.lattice import Lattice
+from oracle.naive import run_naive
+from oracle.tn import coset_network
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 1e-3)])
+@pytest.mark.parametrize("d,B,delta0", [(3, 3, 0.0), (3, 3, 1e-3), (5, 3, 1e-3), (7, 2, 1e-4)])
+def test_partly_filled_passes(precision, tol, d, B, delta0):
+    p, iters = 0.1, 12
+    _, _, S = synth.sample_syndromes(8800 + d, 0, B, d, p)
+    want = np.empty((B, 4))
+    its = np.empty((B, 4), dtype=np.int64)
+    for b in range(B):
+        for c in range(4):
+            want[b, c], _, its[b, c], _ = run_naive(coset_network(Lattice(d), S[b], c, p), 4, iters, 0.1, delta0)
+    first = None
+    for warps, cosets, messages in ((0, 0, 0), (8, 1, 1), (8, 2, 3), (4, 2, 1), (4, 4, 1)):
+        if messages == 3 and precision == "fp64":
+            warps, cosets = 4, 2
+        prm = pkg.DecoderParams(d=d, k=4, p=p, max_iter=iters, delta0=delta0, precision=precision, algorithm="fused",
+                                warps=warps, cosets=cosets, messages=messages)
+        out = pkg.decode(torch.from_numpy(S).cuda(), prm)
+        got = out["logp"].cpu().numpy()
+        same = out["iters"].cpu().numpy() == its          # FP32 may stop an iteration apart at the threshold
+        assert same.mean() >= (1.0 if precision == "fp64" else 0.75)
+        assert np.max(np.abs(got - want)[same]) <= tol, (warps, cosets, messages)
+        if first is None:
+            first = out
+        for key in ("logp", "delta", "iters", "flags", "decision"):
+            assert torch.equal(out[key], first[key]), (warps, cosets, messages, key)
