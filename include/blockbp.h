@@ -105,9 +105,10 @@ extern "C" {
  *             k = 4 at odd d only, where every block is 4 x 4 or one node
  *             wide; small per-warp buffers, sized for more CTAs per SM; for
  *             bbp_decode_mixed only on request, see there).
- *             0 picks the first compiled shape, in order of measured speed,
- *             whose shared memory allows the CTAs per SM its registers are
- *             sized for, else the first that fits; compiled (warps, cosets):
+ *             0 picks by geometry and, for FP32 at k = 4 and odd d, by batch
+ *             size (few syndromes: one coset per CTA); where the geometry's
+ *             messages do not fit in shared memory, workspace slots;
+ *             compiled (warps, cosets):
  *             FP32 (8,4) (8,2) (4,2) (4,4) (16,1) (8,1) (4,1), of which (8,4)
  *             and (8,2) also with workspace messages and in register-form-only
  *             variants ((8,4) sized for 4 and for 3 CTAs per SM, the first

@@ -28,6 +28,19 @@ bool shape_of(const bbp_params* p, const Geo& g, int M, int* warps, int* cosets,
   return ok;
 }
 
+// A launch that asks for no shape takes the kernel measured fastest for its
+// geometry and batch; lean_ok: every syndrome has odd distance.
+void pick_default(const bbp_params* p, const Geo& g, int M, int64_t B, int* warps, int* cosets, bool* gm, int* lean,
+                  bool lean_ok) {
+  if (p->launch_warps != 0 || p->launch_cosets != 0 || (p->launch_messages != 0 && p->launch_messages != 3)) return;
+  if (!lean_ok || g.k != 4 || g.d % 2 == 0) return;
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+    return;
+  if (bbp::fused_pick(p->precision, g, M, B, sms, warps, cosets, lean)) *gm = false;
+}
+
 int check_params(const bbp_params* p) {
   if (!p) return BBP_EINVAL;
   if (p->d < 2 || p->d > 64) return BBP_EINVAL;
@@ -171,8 +184,11 @@ int bbp_decode_batch_ex(const uint8_t* syndromes, int64_t B, const bbp_params* p
   cudaError_t e;
   if (prm->algorithm == BBP_ALG_FUSED) {
     if (s.warps == 0) return BBP_EUNSUPPORTED;
-    e = prm->precision == BBP_FP64 ? bbp::launch_fused_f64(a, s.warps, s.cosets, s.gm, s.lean, st)
-                                   : bbp::launch_fused_f32(a, s.warps, s.cosets, s.gm, s.lean, st);
+    int warps = s.warps, cosets = s.cosets, lean = s.lean;
+    bool gm = s.gm;
+    pick_default(prm, s.g, s.M, B, &warps, &cosets, &gm, &lean, true);
+    e = prm->precision == BBP_FP64 ? bbp::launch_fused_f64(a, warps, cosets, gm, lean, st)
+                                   : bbp::launch_fused_f32(a, warps, cosets, gm, lean, st);
   } else
     e = prm->precision == BBP_FP64 ? bbp::launch_decode_f64(a, st) : bbp::launch_decode_f32(a, st);
   if (e != cudaSuccess) return BBP_ECUDA;
@@ -248,6 +264,7 @@ int bbp_decode_mixed(const uint8_t* syndromes, const int64_t* offsets, const int
   bool gm = false;
   bbp::count_messages(a.geo, 1, &Mmax, &ae);
   if (!shape_of(prm, a.geo, Mmax, &w, &c, &gm, &lean, lean_req)) return BBP_EUNSUPPORTED;
+  pick_default(prm, a.geo, Mmax, B, &w, &c, &gm, &lean, lean_req);
   if (gm) {   // message slots after the counter
     const size_t elem = prm->precision == BBP_FP64 ? sizeof(double) : sizeof(float);
     m.slots = fused_slots(B, c);

@@ -7,6 +7,10 @@ namespace bbp {
 cudaError_t launch_fused_f64(const LaunchArgs& a, int warps, int cosets, bool gm, int lean, cudaStream_t st) {
   if (lean > 0) {                          // every block update in register form, sized for `lean` CTAs per SM
     switch (warps * 100 + cosets * 10 + lean) {
+      case 1611: return launch_fused_nw<double, 16, 1, 4, false, 1>(a, st);
+      case 1621: return launch_fused_nw<double, 16, 2, 4, false, 1>(a, st);
+      case 841: return launch_fused_nw<double, 8, 4, 4, false, 1>(a, st);
+      case 443: return launch_fused_nw<double, 4, 4, 4, false, 3>(a, st);
       case 424: return launch_fused_nw<double, 4, 2, 4, false, 4>(a, st);
       case 822: return launch_fused_nw<double, 8, 2, 4, false, 2>(a, st);
       default: return cudaErrorInvalidValue;
@@ -33,6 +37,10 @@ cudaError_t launch_fused_mixed_f64(const LaunchArgs& a, const MixedLaunch& m, in
                                    int lean, cudaStream_t st) {
   if (lean > 0) {                          // every distance odd: every block update in register form
     switch (warps * 100 + cosets * 10 + lean) {
+      case 1611: return launch_fused_mixed_nw<double, 16, 1, 4, false, 1>(a, m, st);
+      case 1621: return launch_fused_mixed_nw<double, 16, 2, 4, false, 1>(a, m, st);
+      case 841: return launch_fused_mixed_nw<double, 8, 4, 4, false, 1>(a, m, st);
+      case 443: return launch_fused_mixed_nw<double, 4, 4, 4, false, 3>(a, m, st);
       case 424: return launch_fused_mixed_nw<double, 4, 2, 4, false, 4>(a, m, st);
       case 822: return launch_fused_mixed_nw<double, 8, 2, 4, false, 2>(a, m, st);
       default: return cudaErrorInvalidValue;
@@ -131,6 +139,47 @@ bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, in
     }
   }
   return false;
+}
+
+// The kernel of a default launch at k = 4 where every block has a register
+// form, for B syndromes (G = 4 / cosets CTAs each) on sms SMs.  Few
+// syndromes: as many CTAs as SMs allow at one per SM, 16 warps each, so that
+// a half-round of one coset's messages is a single round of passes (d = 11:
+// 1 syndrome 148 us with (8, 4), 74 us with (16, 1); 64 at d = 9: 125 and 78;
+// 152 at d = 11: 170 with (8, 4, 4), 137 with (16, 4, 1)).  Then four cosets per
+// CTA and as many CTAs as shared memory allows: the more warps per CTA the
+// fewer CTAs fit ((8, 4, 4) at d = 11, 3 at 13 and 15, 2 at 17, and from d = 19
+// on one CTA of 16 warps: d = 21, 2000 syndromes 4.64 ms against 5.58 for (8,
+// 4, 2) and 4.93 for (8, 2, 2)).  Small codes have too few passes per
+// half-round for 8 warps: four warps where six such CTAs fit (d <= 9; d = 5,
+// 10^4 syndromes 1.58 ms against 1.78), or five and the batch is long enough
+// to hide its slower CTAs' tail (d = 11, 10^4 syndromes 4.93 ms against 5.06).
+// Where four cosets do not fit (d >= 27), two or one.  FP64 is bound by its
+// pipe, so at large batches the shape matters little ((8, 2, 2) at d = 11, 1000
+// syndromes: 12.2 ms, all others 12.3 to 13.1) but for the smallest codes
+// ((4, 4, 3) at d = 5: 2.20 ms against 3.01); one syndrome 709 us with (16, 1),
+// 1232 with (4, 2).
+bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, int* warps, int* cosets, int* lean) {
+  auto fit = [&](int w, int c) {
+    const int smem = precision == 0 ? fused_smem_for<double, 4>(g, M, w, c, false, true)
+                                    : fused_smem_for<float, 4>(g, M, w, c, false, true);
+    return smem > kMaxSmemBytes ? 0 : kSmemPerSm / (smem + kSmemReservedPerCta);
+  };
+  auto take = [&](int w, int c, int l) { *warps = w; *cosets = c; *lean = l; return true; };
+  int c = 4 * B <= sms ? 1 : (2 * B <= sms ? 2 : 4);
+  while (c > 1 && fit(16, c) < 1) c /= 2;
+  if (fit(16, c) < 1) return false;
+  if (precision == 0) {
+    if (c < 4) return take(16, c, 1);
+    if (B <= sms) return take(8, 4, 1);
+    if (fit(4, 4) >= 6) return take(4, 4, 3);
+    return fit(8, 2) >= 2 ? take(8, 2, 2) : take(16, 2, 1);
+  }
+  if (B <= sms || c < 4 || fit(8, 4) < 2) return take(16, c, 1);
+  if (B <= 2ll * sms) return take(8, 4, 2);
+  if (fit(4, 4) >= 6 || (fit(4, 4) >= 5 && B >= 16ll * sms)) return take(4, 4, 6);
+  const int n = fit(8, 4);
+  return take(8, 4, n < 4 ? n : 4);
 }
 
 }  // namespace bbp

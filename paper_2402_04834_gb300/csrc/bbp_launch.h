@@ -55,6 +55,10 @@ constexpr int kSmemReservedPerCta = 1024;       // reserved by the runtime per r
 bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, int* messages, bool allow_lean = true,
                  int* lean_blocks = nullptr);
 
+// The register-form-only kernel of a default launch (k = 4, odd d) for B
+// syndromes on sms SMs; false where the shape of fused_shape stands.
+bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, int* warps, int* cosets, int* lean);
+
 struct MixedLaunch {
   const int32_t* d_of;
   const int64_t* offsets;

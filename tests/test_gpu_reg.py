@@ -43,3 +43,20 @@ def test_partly_filled_passes(precision, tol, d, B, delta0):
             first = out
         for key in ("logp", "delta", "iters", "flags", "decision"):
             assert torch.equal(out[key], first[key]), (warps, cosets, messages, key)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,B", [(3, 700), (5, 1), (5, 80), (7, 200), (9, 400), (11, 39), (11, 77), (11, 153), (11, 305),
+                                 (11, 2500), (13, 400), (17, 320), (21, 160), (27, 160), (29, 3), (29, 160), (41, 2),
+                                 (53, 2)])
+def test_default_kernel_of_every_size_gives_the_same_bits(d, B):
+    # The default launch takes a kernel by geometry and batch; each gives the
+    # bits of a kernel asked for by shape (messages in shared memory, or in
+    # workspace slots where they do not fit).
+    _, _, S = synth.sample_syndromes(9900 + d, 0, B, d, 0.11)
+    s = torch.from_numpy(S).cuda()
+    base = dict(d=d, k=4, p=0.11, max_iter=6, delta0=2e-3, precision="fp32", algorithm="fused")
+    a = pkg.decode(s, pkg.DecoderParams(**base))
+    b = pkg.decode(s, pkg.DecoderParams(**base, messages=1 if d <= 46 else 2))
+    for key in ("logp", "delta", "iters", "flags", "decision"):
+        assert torch.equal(a[key], b[key]), key
