@@ -1091,7 +1091,11 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   if constexpr (!kLean) ws = fused_ws_at<T, K>(smem + Lo.ws + warp * Lo.ws_stride, G);
 
   const T pI = a.pI_w, pE = a.pE_w;
-  const RegUpd<T> upd{a.eta_w, a.one_m_eta_w, ovl, M};
+  RegUpd<T> upd{a.eta_w, a.one_m_eta_w, T(0), T(0), ovl, M};
+  if constexpr (sizeof(T) == 8) {
+    upd.rho = pI / pE;
+    upd.rho_m1 = (pI - pE) / pE;
+  }
   unsigned act = (1u << G) - 1;                      // cosets still iterating
   for (int it = 1; it <= a.max_iter && M > 0 && act; ++it) {
     int n = 0;

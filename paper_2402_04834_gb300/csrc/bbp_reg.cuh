@@ -227,6 +227,7 @@ struct RegMsgs {
 template <typename T>
 struct RegUpd {
   T eta, one_m_eta;
+  T rho, rho_m1;                            // pi(I) / pi(X), that - 1 (FP64)
   T* ovl;                                   // Delta term of each (coset, message)
   int M;
 };
@@ -256,9 +257,23 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 
 // 1 / sqrt(s), 0 for s = 0: the scale of a unit-norm vector (Remark 3).
 // FP32 takes the hardware reciprocal square root (a scale factor, whose last
-// bit does not matter); FP64 the rounded square root and quotient.
+// bit does not matter).  FP64 refines it by one third-order Newton (Halley)
+// step y + y r (1/2 + 3 r / 8), r = 1 - m y^2, which squares and more the
+// seed's 2^-22: five FP64 operations, where the rounded square root and
+// quotient were most of an update's (FP64 issues two lanes a cycle per SM).
+// The seed is taken of s scaled by an even power of two into [1, 4).
 __device__ __forceinline__ float inv_norm(float s) { return s > 0.f ? rsqrtf(s) : 0.f; }
-__device__ __forceinline__ double inv_norm(double s) { return s > 0.0 ? 1.0 / sqrt(s) : 0.0; }
+__device__ __forceinline__ double inv_norm(double s) {
+  if (!(s > 0.0)) return 0.0;
+  const int hi = __double2hiint(s), e = hi >> 20;          // biased exponent (s > 0)
+  if (e == 0 || e == 0x7ff) return 1.0 / sqrt(s);          // subnormal, infinity
+  const int k = (e - 1023) & ~1;
+  const double m = __hiloint2double(hi - (k << 20), __double2loint(s));
+  const double y = (double)rsqrtf((float)m);
+  const double r = fma(-(m * y), y, 1.0);
+  const double z = fma(y * r, fma(r, 0.375, 0.5), y);
+  return __hiloint2double(__double2hiint(z) - ((k >> 1) << 20), __double2loint(z));
+}
 
 // Coefficient v (0 .. 3) of the qubit in field f of t = ids ^ lane pattern:
 // pI where the field equals v.  With the lane's bit be at the field's beta
@@ -581,6 +596,187 @@ __device__ __forceinline__ void quad_pass(T* stage, T pI, T pE, const RegMsgs<T,
   }
 }
 
+// The update of eight 4 x 4 blocks in FP64, with as few FP64 operations as the
+// structure allows (the FP64 pipe is the bound; selects cost nothing beside
+// it).  A qubit's table is pi(X) everywhere but at its id, so with tables
+// divided by pi(X) (a factor of the message, which the normalisation takes
+// out) a butterfly is the pair's sum, plus (rho - 1) times one of the pair
+// where the id's beta matches: rows share sums, half of the rows need no
+// multiply-add, and of column 1's four (b0, b1) products three are the value
+// itself.  170 operations a lane (four rows) and contraction against 264 for
+// quad_pass's; with inv_norm, 230 against 372 for an update.  1000 syndromes
+// at d = 11, p = 0.10: 16.4 -> 12.6 ms, FP64 pipe 87 % busy.
+template <bool GM>
+__device__ __forceinline__ void quad_update64(double* stage, const RegMsgs<double, GM>& ms,
+                                              const RegJob<double, GM>& jb, int lane, const RegUpd<double>& upd) {
+  using T = double;
+  const int r1 = (lane >> 1) & 1, r3 = lane & 1, g = lane >> 2;
+  const unsigned tq = jb.id ^ (r1 ? 0x0505u : 0u) ^ (r3 ? 0x0484u : 0u);   // as in quad_pass
+  auto beta = [&](int f) { return (bool)((tq >> (2 * f)) & 1u); };
+  auto alpha = [&](int f) { return (bool)((tq >> (2 * f + 1)) & 1u); };
+  const T rho = upd.rho, rm1 = upd.rho_m1;
+  T* sj = stage + (g << 4);
+  {
+    const T* A = ms.at(jb.cq, jb.up());
+    T a[8];                                                // [a1][v][e] of a0 = r3
+    if (jb.srev()) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) a[i] = A[r3 + 2 * (i >> 2) + 4 * ((i >> 1) & 1) + 8 * (i & 1)];
+    } else {
+      T lo[4], hi[4];
+      vcopy4(A + 8 * r3, lo);
+      vcopy4(A + 8 * r3 + 4, hi);
+#pragma unroll
+      for (int i = 0; i < 4; ++i) { a[i] = lo[i]; a[4 + i] = hi[i]; }
+    }
+    // [alpha][q0]: v = 0 and v = 1 of a1 = q0 ^ alpha, e = q0.
+    const T v0[4] = {a[0], a[5], a[4], a[1]}, v1[4] = {a[2], a[7], a[6], a[3]};
+    T c[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c[i] = v0[i] + v1[i];
+    const bool al = alpha(4), be = beta(4);
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const T e = fma(rm1, al ? (be ? v1[2 + q] : v0[2 + q]) : (be ? v1[q] : v0[q]), al ? c[2 + q] : c[q]);
+      c[q] = al ? c[q] : e;
+      c[2 + q] = al ? e : c[2 + q];
+    }
+    vstore4(sj + 8 * r1 + 4 * r3, c);
+  }
+  __syncwarp();
+  const RowAt at(jb.chk0(), r1, r3);
+  T S0[2][2][2];                                           // [a0][q0][q2]
+  {
+    const T* X = ms.at(jb.cq, jb.in());
+    T x[2][2], u[2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) x[a][b] = X[at(a, b)];
+    const bool al = alpha(1);
+    const T k = beta(1) ? 0.0 : rm1;
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      const T s = x[a][0] + x[a][1];
+#pragma unroll
+      for (int b = 0; b < 2; ++b) u[a][b] = fma(k, al ? x[a][b ^ 1] : x[a][b], s);
+    }
+    const bool al0 = alpha(0), be0 = beta(0);
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+      const T s = u[0][b] + u[1][b];
+#pragma unroll
+      for (int a = 0; a < 2; ++a) {
+        const T e = fma(rm1, al0 ? u[a ^ 1][b] : u[a][b], s);
+        S0[0][a][b] = be0 ? s : e;
+        S0[1][a][b] = be0 ? e : s;
+      }
+    }
+  }
+  // The rows with r0 ^ r2 = beta: (r, r ^ beta), r = 0, 1.
+  auto butterfly = [&](int f, const T (&o)[2][2], T (&t)[2][2]) {   // over r1, beta = r0 ^ r2
+    const bool al = alpha(f), be = beta(f);
+    T p[2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        p[a][b] = shx(o[a][b], 2);
+        t[a][b] = o[a][b] + p[a][b];
+      }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const T w = be ? (al ? p[r][r ^ 1] : o[r][r ^ 1]) : (al ? p[r][r] : o[r][r]);
+      const T e = fma(rm1, w, be ? t[r][r ^ 1] : t[r][r]);
+      t[r][r] = be ? t[r][r] : e;
+      t[r][r ^ 1] = be ? e : t[r][r ^ 1];
+    }
+  };
+  // Column 1's lower qubit scales T_h, h = its id's b0, where b1 ^ r2 is its
+  // beta: b1 = beta scales row r2 = 0 (P), b1 = 1 - beta row r2 = 1 (Q); the
+  // other b0 (O) is the same for both b1.
+  const bool h = alpha(3), hv = beta(3);
+  const bool al5 = alpha(5);
+  const T k5 = beta(5) ? 0.0 : rm1;
+  T YO[2][2], YP[2][2], YQ[2][2];
+#pragma unroll
+  for (int a0 = 0; a0 < 2; ++a0) {
+    T cA[4];
+    vcopy4(sj + 8 * r1 + 4 * a0, cA);
+    T t[2][2];
+    butterfly(2, S0[a0], t);
+    T uO[2][2], uP[2][2], uQ[2][2];
+#pragma unroll
+    for (int a = 0; a < 2; ++a) {
+      T th[2], to[2], rh[2];
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        th[b] = __shfl_sync(kFull, t[a][b], (lane & ~1) | (h ? 1 : 0));
+        to[b] = __shfl_sync(kFull, t[a][b], (lane & ~1) | (h ? 0 : 1));
+        rh[b] = rho * th[b];
+      }
+      const T sO = to[0] + to[1], sP = rh[0] + th[1], sQ = th[0] + rh[1];
+      uO[a][0] = fma(k5, al5 ? to[1] : to[0], sO);
+      uO[a][1] = fma(k5, al5 ? to[0] : to[1], sO);
+      uP[a][0] = fma(k5, al5 ? th[1] : rh[0], sP);
+      uP[a][1] = fma(k5, al5 ? rh[0] : th[1], sP);
+      uQ[a][0] = fma(k5, al5 ? rh[1] : th[0], sQ);
+      uQ[a][1] = fma(k5, al5 ? th[0] : rh[1], sQ);
+    }
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        if (a0 == 0) {
+          YO[a][b] = fma(cA[a], uO[a][b], cA[2 + a] * uO[a ^ 1][b]);
+          YP[a][b] = fma(cA[a], uP[a][b], cA[2 + a] * uP[a ^ 1][b]);
+          YQ[a][b] = fma(cA[a], uQ[a][b], cA[2 + a] * uQ[a ^ 1][b]);
+        } else {
+          YO[a][b] = fma(cA[a], uO[a][b], fma(cA[2 + a], uO[a ^ 1][b], YO[a][b]));
+          YP[a][b] = fma(cA[a], uP[a][b], fma(cA[2 + a], uP[a ^ 1][b], YP[a][b]));
+          YQ[a][b] = fma(cA[a], uQ[a][b], fma(cA[2 + a], uQ[a ^ 1][b], YQ[a][b]));
+        }
+      }
+  }
+  T uu[2][2];
+  {
+    const T* B = ms.at(jb.cq, jb.lo());
+    T bm[2][2][2];                                         // B[b0 b1 r3 ff]
+    if (jb.srev()) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) bm[i >> 2][(i >> 1) & 1][i & 1] = B[(i >> 2) + 2 * ((i >> 1) & 1) + 4 * r3 + 8 * (i & 1)];
+    } else {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) bm[i >> 2][(i >> 1) & 1][i & 1] = B[4 * (i >> 1) + 2 * r3 + (i & 1)];
+    }
+    T S2[2][2][2];                                         // [ff][q0][q2]
+#pragma unroll
+    for (int f = 0; f < 2; ++f) {
+      const T bO = (h ? bm[0][0][f] : bm[1][0][f]) + (h ? bm[0][1][f] : bm[1][1][f]);
+      const T b0 = h ? bm[1][0][f] : bm[0][0][f], b1 = h ? bm[1][1][f] : bm[0][1][f];
+      const T bP = hv ? b1 : b0, bQ = hv ? b0 : b1;
+#pragma unroll
+      for (int a = 0; a < 2; ++a)
+#pragma unroll
+        for (int b = 0; b < 2; ++b) S2[f][a][b] = fma(bQ, YQ[a][b], fma(bP, YP[a][b], bO * YO[a][b]));
+    }
+    const bool al = alpha(7), be = beta(7);
+#pragma unroll
+    for (int a = 0; a < 2; ++a)
+#pragma unroll
+      for (int b = 0; b < 2; ++b) {
+        const T z0 = S2[0][a][b], z1 = S2[1][a][b];
+        const T p0 = shx(z0, 1), p1 = shx(z1, 1);
+        const bool one = be != (b == 1);                   // the id's beta against r2: z1 or z0
+        uu[a][b] = fma(rm1, one ? (al ? p1 : z1) : (al ? p0 : z0), (z0 + p0) + (z1 + p1));
+      }
+  }
+  T out[2][2];
+  butterfly(6, uu, out);
+  reg_update16(out, ms, jb, at, (lane & 3) == 0, upd);
+  __syncwarp();
+}
+
 // Eight blocks of one column of 4 nodes: as quad_pass's column 0, both side
 // messages have one leg.
 template <typename T, bool GM, bool UPD>
@@ -745,7 +941,8 @@ __device__ __forceinline__ void dot_pass(T* stage, T pI, T pE, const RegMsgs<T, 
 template <typename T, bool GM, bool UPD, int SHAPE>
 __device__ __forceinline__ void reg_pass(T* stage, T pI, T pE, const RegMsgs<T, GM>& ms, const RegJob<T, GM>& jb,
                                          int lane, const RegUpd<T>& upd) {
-  if constexpr (SHAPE == kShapeQuad) quad_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
+  if constexpr (SHAPE == kShapeQuad && UPD && sizeof(T) == 8) quad_update64<GM>(stage, ms, jb, lane, upd);
+  else if constexpr (SHAPE == kShapeQuad) quad_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
   else if constexpr (SHAPE == kShapeCol) col_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
   else if constexpr (SHAPE == kShapeRow) row_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
   else dot_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
