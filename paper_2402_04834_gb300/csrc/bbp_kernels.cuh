@@ -74,6 +74,30 @@ __device__ __forceinline__ T group_sum(T v, int G) {
   return v;
 }
 
+// 1 / sqrt(s), 0 for s = 0: the scale of a unit-norm vector (Remark 3).
+// FP32 takes the hardware reciprocal square root (a scale factor, whose last
+// bit does not matter).  FP64 refines it by one third-order Newton (Halley)
+// step y + y r (1/2 + 3 r / 8), r = 1 - m y^2, which squares and more the
+// seed's 2^-22: five FP64 operations, where the rounded square root and
+// quotient were most of an update's (FP64 issues two lanes a cycle per SM).
+// The seed is taken of s scaled by an even power of two into [1, 4).
+__device__ __forceinline__ float inv_norm(float s) { return s > 0.f ? rsqrtf(s) : 0.f; }
+// Reciprocal square root of m in [1, 4).
+__device__ __forceinline__ double rsqrt_unit(double m) {
+  const double y = (double)rsqrtf((float)m);
+  const double r = fma(-(m * y), y, 1.0);
+  return fma(y * r, fma(r, 0.375, 0.5), y);
+}
+__device__ __forceinline__ double inv_norm(double s) {
+  if (!(s > 0.0)) return 0.0;
+  const int hi = __double2hiint(s), e = hi >> 20;          // biased exponent (s > 0)
+  if (e == 0 || e == 0x7ff) return 1.0 / sqrt(s);          // subnormal, infinity
+  const int k = (e - 1023) & ~1;
+  const double m = __hiloint2double(hi - (k << 20), __double2loint(s));
+  const double z = rsqrt_unit(m);
+  return __hiloint2double(__double2hiint(z) - ((k >> 1) << 20), __double2loint(z));
+}
+
 // Per-warp shared-memory workspace.  SITE holds one (2D) x 2 x (2D) site.
 template <typename T, int K, int DM>
 struct WarpWS {
@@ -488,6 +512,299 @@ __device__ __noinline__ void svd_step(WarpWS<T, K, DM>& ws, const Ctx<T, K>& c, 
   __syncwarp();
 }
 
+// ---------------------------------------------------------------------------
+// The two steps in FP64.  The FP64 pipe (two lanes a cycle per SM) is all
+// that bounds them, so they are written for few FP64 operations: element i of
+// a row or column sits in half-lane i % 2, place i / 2, and loops stop at the
+// matrix's own size (four places at a time) instead of the capacity; compares
+// of non-negative values run on their bits; square roots and quotients are
+// hardware seeds refined in a few operations, where the library's were more
+// than half of a step.
+
+// x > y and x < y for non-negative x, y (no NaN), on the integer pipe.
+__device__ __forceinline__ bool pos_gt(double x, double y) { return __double_as_longlong(x) > __double_as_longlong(y); }
+__device__ __forceinline__ bool pos_lt(double x, double y) { return pos_gt(y, x); }
+
+// lq_step: modified Gram-Schmidt as there (two passes, the same dependence
+// test), with unnormalised rows: the products <x_i, x_j> of a step give the
+// norm of row j too, and rows are scaled once at the end of a pass.
+template <int K, int DM>
+__device__ __noinline__ void lq_step64(WarpWS<double, K, DM>& ws, int s, int lane) {
+  constexpr int HC = 2 * DM;                 // places per half-row
+  static_assert(HC % 4 == 0, "places are taken four at a time");
+  const int pl = ws.bond[s], pr = ws.bond[s + 1];
+  const int nc = 2 * pr;                     // row length (<= 4D), even
+  const int row = lane & 15, half = lane >> 4;
+  const bool own = row < pl;
+  const int tb = nc >> 1;                    // places in use
+  double x[HC];
+  const double* A = ws.psi[s];
+#pragma unroll
+  for (int t = 0; t < HC; ++t) x[t] = (own && t < tb) ? A[row * nc + 2 * t + half] : 0.0;
+  double nrm0 = 0;
+#pragma unroll
+  for (int c = 0; c < HC; c += 4)
+    if (c < tb) {
+#pragma unroll
+      for (int t = c; t < c + 4; ++t) nrm0 = fma(x[t], x[t], nrm0);
+    }
+  nrm0 += __shfl_xor_sync(kFull, nrm0, 16);
+  double* L1 = ws.mat;                       // [pass][a][j] coefficients, pl x pl each
+  double* L2 = ws.mat + 4 * DM * DM;
+  for (int e = lane; e < 2 * 4 * DM * DM; e += 32) ws.mat[e] = 0.0;
+  __syncwarp();
+  const double tau2 = GsTau<double>::v() * GsTau<double>::v();
+  const double ref = tau2 * nrm0;
+  unsigned kept = 0;                         // bit j set: q_j is a row of Q
+  for (int pass = 0; pass < 2; ++pass) {
+    double* Lc = pass == 0 ? L1 : L2;
+    double scale = 0.0;                      // of this lane's row
+    for (int j = 0; j < pl; ++j) {
+      if (pass == 1 && !((kept >> j) & 1u)) continue;      // zero row
+      double q[HC], cf = 0;
+#pragma unroll
+      for (int c = 0; c < HC; c += 4)
+        if (c < tb) {
+#pragma unroll
+          for (int t = c; t < c + 4; ++t) {
+            q[t] = __shfl_sync(kFull, x[t], j + 16 * half);
+            cf = fma(x[t], q[t], cf);
+          }
+        }
+      cf += __shfl_xor_sync(kFull, cf, 16);
+      const double nj2 = __shfl_sync(kFull, cf, j);
+      const bool indep = pos_gt(nj2, pass == 0 ? __shfl_sync(kFull, ref, j) : 0.0) && pos_gt(nj2, 0.0);
+      if (!indep) {                          // dependent on the earlier rows: dropped, its coefficients stay
+        if (row == j) {
+#pragma unroll
+          for (int t = 0; t < HC; ++t) x[t] = 0.0;
+        }
+        continue;
+      }
+      if (pass == 0) kept |= 1u << j;
+      const double rs = inv_norm(nj2);
+      const double lj = cf * rs;             // <x_row, q_j>; of row j its norm
+      if (row == j) scale = rs;
+      if (own && row >= j && half == 0) Lc[row * pl + j] = lj;
+      const double f = (own && row > j) ? -(lj * rs) : 0.0;
+#pragma unroll
+      for (int c = 0; c < HC; c += 4)
+        if (c < tb) {
+#pragma unroll
+          for (int t = c; t < c + 4; ++t) x[t] = fma(f, q[t], x[t]);
+        }
+    }
+#pragma unroll
+    for (int c = 0; c < HC; c += 4)
+      if (c < tb) {
+#pragma unroll
+        for (int t = c; t < c + 4; ++t) x[t] *= scale;
+      }
+  }
+  __syncwarp();
+  // Compact the kept rows: Q (r x nc) into site s.
+  if (kept == 0u) {          // zero site: keep one (zero) row so every bond stays >= 1
+    kept = 1u;
+    if (row == 0) {
+#pragma unroll
+      for (int t = 0; t < HC; ++t) x[t] = 0.0;
+    }
+  }
+  const int r = __popc(kept);
+  const int myidx = __popc(kept & ((1u << row) - 1u));
+  double* Q = ws.psi[s];
+  if (own && ((kept >> row) & 1u)) {
+#pragma unroll
+    for (int t = 0; t < HC; ++t)
+      if (t < tb) Q[myidx * nc + 2 * t + half] = x[t];
+  }
+  // L = L1 * L2 restricted to kept columns: L[a][k] (pl x r) into vm (both
+  // factors are lower triangular).
+  double* Lm = ws.vm;
+  const FastDiv dr(r);
+  for (int e = lane; e < pl * r; e += 32) {
+    const int aa = dr.quo(e), kk = e - aa * r;
+    const int j2 = (int)__fns(kept, 0, kk + 1);
+    double acc = 0;
+    for (int j = j2; j <= aa; ++j) acc += L1[aa * pl + j] * L2[j * pl + j2];
+    Lm[e] = acc;
+  }
+  __syncwarp();
+  // Site s-1 <- site s-1 * L.
+  const int bl = ws.bond[s - 1];
+  double* out = ws.tmp;
+  const double* P = ws.psi[s - 1];
+  for (int e = lane; e < bl * 2 * r; e += 32) {
+    const int rr = dr.quo(e), kk = e - rr * r;
+    double acc = 0;
+    for (int aa = 0; aa < pl; ++aa) acc += P[rr * pl + aa] * Lm[aa * r + kk];
+    out[e] = acc;
+  }
+  __syncwarp();
+  warp_copy(ws.psi[s - 1], out, bl * 2 * r, lane);
+  if (lane == 0) ws.bond[s] = r;
+  __syncwarp();
+}
+
+// svd_step: one-sided Jacobi on the site matrix A (m x n) or, when m < n, on
+// its transpose, so that the q = min(m, n) columns it rotates are the fewer
+// (site 0 has m = 2 rows per left bond).  A pair's rotation solves c t^2 + (b
+// - a) t - c = 0 (a, b the squared norms, c the product) by an FP32 root and
+// one Newton step whose residual is FP64; the cosine is an exact unit-norm
+// scale of that t, so the rotation is orthogonal to rounding whatever t's
+// last bits are.  m >= n: U are the scaled columns, S V^T = U^T A.  m < n: the
+// columns are S V^T and the accumulated rotations U.
+template <int K, int DM>
+__device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<double, K>& c, int s, int lane) {
+  static_assert(DM <= 8 && DM % 4 == 0, "register Jacobi holds at most 16 columns");
+  const int pl = ws.bond[s], pr = ws.bond[s + 1];
+  const int m = 2 * pl, n = pr;
+  const bool tr = m < n;
+  const int q = tr ? m : n, p = tr ? n : m;  // columns, their length
+  const int col = lane & 15, half = lane >> 4;
+  const bool on = col < q;
+  const int tb = (p + 1) >> 1, vb = tr ? (q + 1) >> 1 : 0;
+  double a[DM], v[DM];
+  const double* S = ws.psi[s];
+#pragma unroll
+  for (int t = 0; t < DM; ++t) {
+    const int i = 2 * t + half;
+    a[t] = (on && i < p) ? (tr ? S[col * n + i] : S[i * n + col]) : 0.0;
+    v[t] = (on && i == col) ? 1.0 : 0.0;
+  }
+  auto norm2 = [&]() {                       // of this lane's column
+    double w = 0;
+#pragma unroll
+    for (int e = 0; e < DM; e += 4)
+      if (e < tb) {
+#pragma unroll
+        for (int t = e; t < e + 4; ++t) w = fma(a[t], a[t], w);
+      }
+    return w + __shfl_xor_sync(kFull, w, 16);
+  };
+  double own = norm2();
+  double fro = own;                          // over the 16 columns (each half holds every norm)
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) fro += __shfl_xor_sync(kFull, fro, o);
+  const double eps = Eps<double>::v();
+  const double tol2 = 16.0 * eps * eps * m;
+  const double thr2 = c.cutoff2 * fro / (16.0 * n);
+  const double noise2 = eps * eps * fro / 256.0;
+  const int np = (q + 1) & ~1;
+  if (q >= 2) {
+    for (int sweep = 0; sweep < kMaxSweeps; ++sweep) {
+      bool rotated = false;
+      for (int rnd = 0; rnd < np - 1; ++rnd) {
+        const int pj = on ? rr_partner(col, rnd, np) : col;
+        const int src = (pj & 15) | (half << 4);
+        double pa[DM], cr = 0;
+#pragma unroll
+        for (int e = 0; e < DM; e += 4)
+          if (e < tb) {
+#pragma unroll
+            for (int t = e; t < e + 4; ++t) {
+              pa[t] = __shfl_sync(kFull, a[t], src);
+              cr = fma(a[t], pa[t], cr);
+            }
+          }
+        cr += __shfl_xor_sync(kFull, cr, 16);
+        const double oth = __shfl_sync(kFull, own, src);
+        const bool lo = col < pj;
+        const double al = lo ? own : oth, be = lo ? oth : own;
+        const bool act = on && pj < q && pj != col;
+        const bool skip = (pos_lt(al, thr2) && pos_lt(be, thr2)) || pos_lt(al, noise2) || pos_lt(be, noise2);
+        const bool rot = act && !skip && pos_gt(cr * cr, tol2 * (al * be));
+        if (!__any_sync(kFull, rot)) continue;
+        double cs = 1.0, sn = 0.0;
+        if (rot) {
+          // Scaled by a power of two so that FP32 holds them.
+          const int ex = (1023 << 20) - (max(__double2hiint(al), __double2hiint(be)) & 0x7ff00000);
+          const double sc = __hiloint2double((1023 << 20) + max(-(1000 << 20), min(1000 << 20, ex)), 0);
+          const double d = (be - al) * sc, cc = cr * sc;
+          const float df = (float)d, cf = (float)cc, z = df / (2.f * cf), az = fabsf(z);
+          const float tf = copysignf(az > 1e4f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(az, az, 1.f))), z);
+          const double t0 = (double)tf;
+          const double res = fma(fma(cc, t0, d), t0, -cc);
+          const double t1 = t0 - (double)((float)res / fmaf(2.f * cf, tf, df));
+          cs = rsqrt_unit(fma(t1, t1, 1.0));
+          sn = lo ? -(cs * t1) : cs * t1;
+          rotated = true;
+        }
+#pragma unroll
+        for (int e = 0; e < DM; e += 4)
+          if (e < tb) {
+#pragma unroll
+            for (int t = e; t < e + 4; ++t) a[t] = fma(sn, pa[t], cs * a[t]);
+          }
+#pragma unroll
+        for (int e = 0; e < DM; e += 4)
+          if (e < vb) {
+#pragma unroll
+            for (int t = e; t < e + 4; ++t) v[t] = fma(sn, __shfl_sync(kFull, v[t], src), cs * v[t]);
+          }
+        own = norm2();
+      }
+      if (!__any_sync(kFull, rotated)) break;
+    }
+  }
+  // Squared singular values, their order and the kept count, as in svd_step.
+  const double sq = on ? own : -1.0;
+  int rank = 0;
+  double smax = 0;
+  for (int i = 0; i < q; ++i) {
+    const double si = __shfl_sync(kFull, sq, i);
+    rank += (si > sq || (si == sq && i < col)) ? 1 : 0;
+    smax = si > smax ? si : smax;
+  }
+  const double floor2 = c.cutoff2 * smax > noise2 ? c.cutoff2 * smax : noise2;
+  const int keep = __popc(__ballot_sync(kFull, half == 0 && sq > floor2));
+  int r = imin(imin(keep, c.D), m);
+  if (r < 1) r = 1;
+  __syncwarp();
+  double* U = ws.mat;                        // m x r
+  double* svt = ws.mat + 2 * DM * DM;        // r x n
+  const FastDiv dn(n);
+  if (on && rank < r) {
+    const double inv = tr ? 1.0 : inv_norm(sq);
+#pragma unroll
+    for (int t = 0; t < DM; ++t) {
+      const int i = 2 * t + half;
+      if (tr) {
+        if (i < n) svt[rank * n + i] = a[t];
+        if (i < m) U[i * r + rank] = v[t];
+      } else {
+        if (i < m) U[i * r + rank] = a[t] * inv;
+      }
+    }
+  }
+  __syncwarp();
+  if (!tr) {
+    for (int e = lane; e < r * n; e += 32) {
+      const int kk = dn.quo(e), jj = e - kk * n;
+      double acc = 0;
+      for (int i = 0; i < m; ++i) acc = fma(U[i * r + kk], S[i * n + jj], acc);
+      svt[e] = acc;
+    }
+    __syncwarp();
+  }
+  // Site s <- U (m x r) row-major as (pl, 2, r); site s+1 <- (S V^T) * site s+1.
+  warp_copy(ws.psi[s], U, m * r, lane);
+  const int nx = 2 * ws.bond[s + 2];
+  const double* B = ws.psi[s + 1];
+  double* out = ws.tmp;
+  const FastDiv dnx(nx);
+  for (int e = lane; e < r * nx; e += 32) {
+    const int kk = dnx.quo(e), qq = e - kk * nx;
+    double acc = 0;
+    for (int b = 0; b < n; ++b) acc += svt[kk * n + b] * B[b * nx + qq];
+    out[e] = acc;
+  }
+  __syncwarp();
+  warp_copy(ws.psi[s + 1], out, r * nx, lane);
+  if (lane == 0) ws.bond[s + 1] = r;
+  __syncwarp();
+}
+
 // Divide the last site by its Frobenius norm; return log(norm) when
 // want_log (only the read-out keeps the scale; the log is an FP64 call,
 // which GB300 issues at 1/64 of the FP32 rate), else 0.
@@ -512,8 +829,13 @@ __device__ double normalize_last(WarpWS<T, K, DM>& ws, int h, int lane, bool wan
 // when want_log.
 template <typename T, int K, int DM>
 __device__ __noinline__ double compress(WarpWS<T, K, DM>& ws, const Ctx<T, K>& c, int h, int lane, bool want_log) {
-  for (int s = h - 1; s >= 1; --s) lq_step(ws, s, lane);
-  for (int s = 0; s + 1 < h; ++s) svd_step(ws, c, s, lane);
+  if constexpr (sizeof(T) == 8) {
+    for (int s = h - 1; s >= 1; --s) lq_step64(ws, s, lane);
+    for (int s = 0; s + 1 < h; ++s) svd_step64(ws, c, s, lane);
+  } else {
+    for (int s = h - 1; s >= 1; --s) lq_step(ws, s, lane);
+    for (int s = 0; s + 1 < h; ++s) svd_step(ws, c, s, lane);
+  }
   return normalize_last(ws, h, lane, want_log);
 }
 

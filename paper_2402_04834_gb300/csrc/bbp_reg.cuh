@@ -255,26 +255,6 @@ __device__ __forceinline__ T shx(T v, int mask) { return __shfl_xor_sync(kFull, 
 __device__ __forceinline__ float radd(float a, float b) { return __fadd_rn(a, b); }
 __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a, b); }
 
-// 1 / sqrt(s), 0 for s = 0: the scale of a unit-norm vector (Remark 3).
-// FP32 takes the hardware reciprocal square root (a scale factor, whose last
-// bit does not matter).  FP64 refines it by one third-order Newton (Halley)
-// step y + y r (1/2 + 3 r / 8), r = 1 - m y^2, which squares and more the
-// seed's 2^-22: five FP64 operations, where the rounded square root and
-// quotient were most of an update's (FP64 issues two lanes a cycle per SM).
-// The seed is taken of s scaled by an even power of two into [1, 4).
-__device__ __forceinline__ float inv_norm(float s) { return s > 0.f ? rsqrtf(s) : 0.f; }
-__device__ __forceinline__ double inv_norm(double s) {
-  if (!(s > 0.0)) return 0.0;
-  const int hi = __double2hiint(s), e = hi >> 20;          // biased exponent (s > 0)
-  if (e == 0 || e == 0x7ff) return 1.0 / sqrt(s);          // subnormal, infinity
-  const int k = (e - 1023) & ~1;
-  const double m = __hiloint2double(hi - (k << 20), __double2loint(s));
-  const double y = (double)rsqrtf((float)m);
-  const double r = fma(-(m * y), y, 1.0);
-  const double z = fma(y * r, fma(r, 0.375, 0.5), y);
-  return __hiloint2double(__double2hiint(z) - ((k >> 1) << 20), __double2loint(z));
-}
-
 // Coefficient v (0 .. 3) of the qubit in field f of t = ids ^ lane pattern:
 // pI where the field equals v.  With the lane's bit be at the field's beta
 // position, the field is (alpha, beta ^ be): g[0][be], g[1][be] are
