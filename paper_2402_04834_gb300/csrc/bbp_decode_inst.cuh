@@ -8,12 +8,12 @@
 namespace bbp {
 
 template <typename T>
-int smem_bytes_for(const Geo& g, int M) {
-  return cta_layout(g, M, kMaxK, kWarps, (int)sizeof(WarpWS<T, kMaxK, kMaxD>)).total;
+int smem_bytes_for(const Geo& g, int M, int warps = kWarps) {
+  return cta_layout(g, M, kMaxK, warps, (int)sizeof(WarpWS<T, kMaxK, kMaxD>)).total;
 }
 
-template <typename T>
-cudaError_t launch_decode_t(const LaunchArgs& a, cudaStream_t st) {
+template <typename T, int NW>
+cudaError_t launch_decode_nw(const LaunchArgs& a, cudaStream_t st) {
   KArgs<T> k;
   k.geo = a.geo; k.M = a.M; k.D = a.D; k.max_iter = a.max_iter; k.arena_elems = a.arena_elems;
   k.p = a.p; k.eta = a.eta; k.delta0 = a.delta0; k.delta1 = a.delta1; k.cutoff = a.cutoff;
@@ -22,13 +22,38 @@ cudaError_t launch_decode_t(const LaunchArgs& a, cudaStream_t st) {
   k.init_msgs = nullptr; k.final_msgs = nullptr;
   k.n_items = 0; k.slot_elems = 0;
   set_working(k);
-  const int smem = smem_bytes_for<T>(a.geo, a.M);
-  auto kern = decode_kernel<T, kMaxK, kMaxD, kWarps>;
+  const int smem = smem_bytes_for<T>(a.geo, a.M, NW);
+  auto kern = decode_kernel<T, kMaxK, kMaxD, NW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   const unsigned grid = (unsigned)(a.B * 4);
-  kern<<<grid, kWarps * 32, smem, st>>>(k);
+  kern<<<grid, NW * 32, smem, st>>>(k);
   return cudaGetLastError();
+}
+
+// Warps per CTA (one message update each): eight where they fit beside the
+// tables (the linear algebra is a chain of short dependent steps; one SM holds
+// 8 warps in FP64 either way, 16 instead of 12 in FP32), four for small
+// networks in FP64 unless SMs would stay idle (half-rounds of few messages),
+// sixteen in FP32 for batches that leave SMs idle.  FP64 d = 11: 24 syndromes
+// 285 -> 224 ms, 60: 440 -> 385; d = 5 with k = 3: 60 syndromes 19.1 ms with
+// four, 20.6 with eight, 10 syndromes 12.4 and 10.2.  FP32 d = 11: 24 syndromes
+// 95 ms with four, 59 with eight, 50 with sixteen; 300: 421, 368, 379.
+template <typename T>
+cudaError_t launch_decode_t(const LaunchArgs& a, cudaStream_t st) {
+  int dev = 0, sms = 0;
+  cudaError_t e;
+  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
+  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
+  const bool idle = 4 * a.B <= sms;
+  auto fits = [&](int warps) { return smem_bytes_for<T>(a.geo, a.M, warps) <= kMaxSmemBytes; };
+  if constexpr (sizeof(T) == 4) {
+    if (idle && fits(16)) return launch_decode_nw<T, 16>(a, st);
+    if (fits(8)) return launch_decode_nw<T, 8>(a, st);
+  } else {
+    if ((idle || a.M >= 40) && fits(8)) return launch_decode_nw<T, 8>(a, st);
+  }
+  return launch_decode_nw<T, kWarps>(a, st);
 }
 
 template <typename T, int K>
