@@ -29,16 +29,19 @@ bool shape_of(const bbp_params* p, const Geo& g, int M, int* warps, int* cosets,
 }
 
 // A launch that asks for no shape takes the kernel measured fastest for its
-// geometry and batch; lean_ok: every syndrome has odd distance.
+// geometry and batch.  lean_ok: every syndrome is known to have odd distance;
+// mixed: smaller distances share the launch, so kernels whose buffers depend
+// on more than the largest one's size (k = 5, 6) are left out.
 void pick_default(const bbp_params* p, const Geo& g, int M, int64_t B, int* warps, int* cosets, bool* gm, int* lean,
-                  bool lean_ok) {
-  if (p->launch_warps != 0 || p->launch_cosets != 0 || (p->launch_messages != 0 && p->launch_messages != 3)) return;
-  if (!lean_ok || g.k != 4 || g.d % 2 == 0) return;
+                  bool lean_ok, bool mixed) {
+  if (p->launch_warps != 0 || p->launch_cosets != 0 || (p->launch_messages != 0 && p->launch_messages != (g.k > 4 ? 2 : 3)))
+    return;
+  if (g.k < 4 || (g.k == 4 && (!lean_ok || g.d % 2 == 0)) || (g.k > 4 && mixed)) return;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return;
-  if (bbp::fused_pick(p->precision, g, M, B, sms, warps, cosets, lean)) *gm = false;
+  if (bbp::fused_pick(p->precision, g, M, B, sms, warps, cosets, lean)) *gm = g.k > 4;
 }
 
 int check_params(const bbp_params* p) {
@@ -186,7 +189,7 @@ int bbp_decode_batch_ex(const uint8_t* syndromes, int64_t B, const bbp_params* p
     if (s.warps == 0) return BBP_EUNSUPPORTED;
     int warps = s.warps, cosets = s.cosets, lean = s.lean;
     bool gm = s.gm;
-    pick_default(prm, s.g, s.M, B, &warps, &cosets, &gm, &lean, true);
+    pick_default(prm, s.g, s.M, B, &warps, &cosets, &gm, &lean, true, false);
     e = prm->precision == BBP_FP64 ? bbp::launch_fused_f64(a, warps, cosets, gm, lean, st)
                                    : bbp::launch_fused_f32(a, warps, cosets, gm, lean, st);
   } else
@@ -264,7 +267,7 @@ int bbp_decode_mixed(const uint8_t* syndromes, const int64_t* offsets, const int
   bool gm = false;
   bbp::count_messages(a.geo, 1, &Mmax, &ae);
   if (!shape_of(prm, a.geo, Mmax, &w, &c, &gm, &lean, lean_req)) return BBP_EUNSUPPORTED;
-  pick_default(prm, a.geo, Mmax, B, &w, &c, &gm, &lean, lean_req);
+  pick_default(prm, a.geo, Mmax, B, &w, &c, &gm, &lean, lean_req, true);
   if (gm) {   // message slots after the counter
     const size_t elem = prm->precision == BBP_FP64 ? sizeof(double) : sizeof(float);
     m.slots = fused_slots(B, c);

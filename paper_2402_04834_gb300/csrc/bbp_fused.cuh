@@ -28,6 +28,7 @@
 #pragma once
 
 #include "bbp_kernels.cuh"
+#include "bbp_block6.cuh"
 #include "bbp_reg.cuh"
 
 namespace bbp {
@@ -55,20 +56,30 @@ struct FusedWS {   // (sizes for block side K: slot = FusedDim<K>::slot, vec = F
   T* mb;   // side message B in consumption order, vec per coset
 };
 
-// lean: every block update of the kernel runs in register form (k = 4,
-// every block 4 x 4 or one node wide), whose staging is all a warp needs.
-template <typename T, int K>
-BBP_HD int fused_ws_bytes(int G, bool lean = false) {
-  if (lean) return align_up((int)sizeof(T) * kRegStage, 16);
-  return align_up((int)sizeof(T) * G * (2 * FusedDim<K>::slot + 16 + 2 * FusedDim<K>::vec), 16);
+// Entries of a state buffer.  lean at k = 4: every block update of the
+// kernel runs in register form, whose staging is all a warp needs.  lean at
+// k = 5, 6: full 6 x 6 blocks are updated column by column in registers
+// (bbp_block6.cuh), so the buffers need only hold that form's states and the
+// node-by-node states of the partial blocks; the read-out, which contracts
+// full blocks node by node, takes full-size buffers from the same memory with
+// fewer warps.
+template <int K>
+BBP_HD int fused_slot(const Geo& g, bool lean) {
+  if (K <= 4 || !lean) return FusedDim<K>::slot;
+  return g.k == 6 && g.W % 6 == 5 ? 2 * kBlock6Buf : kBlock6Buf;   // a 6 x 5 block's widest state has 2^11 entries
 }
 
 template <typename T, int K>
-__device__ __forceinline__ FusedWS<T> fused_ws_at(unsigned char* base, int G) {
+BBP_HD int fused_ws_bytes(const Geo& g, int G, bool lean = false) {
+  if (K == 4 && lean) return align_up((int)sizeof(T) * kRegStage, 16);
+  return align_up((int)sizeof(T) * G * (2 * fused_slot<K>(g, lean) + 16 + 2 * FusedDim<K>::vec), 16);
+}
+
+template <typename T, int K>
+__device__ __forceinline__ FusedWS<T> fused_ws_at(unsigned char* base, int G, int slot) {
   static_assert(K != 4 || kRegStage <= FusedDim<K>::slot, "the staging fits in a state buffer");
   FusedWS<T> w;
   T* p = reinterpret_cast<T*>(base);
-  const int slot = FusedDim<K>::slot;
   w.s0 = p;
   w.s1 = p + G * slot;
   w.wn = p + 2 * G * slot;
@@ -102,8 +113,8 @@ BBP_HD FusedLayout fused_layout(const Geo& g, int M, int nwarps, int G, bool gm 
   FusedLayout L;
   int o = 0;
   L.parity = o; o = align_up(o + 2 * g.d * 8, 16);             // the pure error, as prefix parities
-  L.frame = o;  if (!lean) o = align_up(o + G * g.W * g.W, 16);
-  L.msg_of = o; if (!lean) o = align_up(o + 2 * g.nb * g.nb * 4, 16);
+  L.frame = o;  if (!lean || K > 4) o = align_up(o + G * g.W * g.W, 16);
+  L.msg_of = o; if (!lean || K > 4) o = align_up(o + 2 * g.nb * g.nb * 4, 16);
   L.meta = o;   o = align_up(o + 2 * M, 16);
   L.work = o;   o = align_up(o + 2 * M, 16);                   // lists of both colours
   L.ovl = o;    o = align_up(o + (int)sizeof(T) * G * M, 16);
@@ -117,7 +128,7 @@ BBP_HD FusedLayout fused_layout(const Geo& g, int M, int nwarps, int G, bool gm 
   L.msgs = o;   // the messages, unless they live in the workspace
   if (!gm) o = align_up(o + (int)sizeof(T) * G * fused_coset_stride<K>(M, gm), 16);
   L.ws = o;
-  L.ws_stride = fused_ws_bytes<T, K>(G, lean);
+  L.ws_stride = fused_ws_bytes<T, K>(g, G, lean);
   o = align_up(o + nwarps * L.ws_stride, 16);
   L.total = o;
   return L;
@@ -745,6 +756,42 @@ __device__ __forceinline__ void fused_sweep_body(const FusedWS<T>& ws, const Ctx
   }
 }
 
+// The outgoing vector of a full 6 x 6 block (one coset) into ws.s0, as
+// fused_sweep leaves it.
+template <typename T, int K>
+__device__ __forceinline__ void block6_update(const FusedWS<T>& ws, const Ctx<T, K>& c, const T* msgs, const Frame& f,
+                                              int lane) {
+  constexpr int VEC = FusedDim<K>::vec;
+  Block6<T> k;
+  int i0, j0;
+  f.node(0, 0, &i0, &j0);
+  k.chk0 = (i0 + j0) & 1;
+  // Side messages in consumption order; the qubits' ids, one per lane.
+#pragma unroll
+  for (int u = 0; u < 2; ++u) {
+    const int i = lane + 32 * u, j = f.rev ? bitrev(i, 6) : i;
+    if (f.a_idx >= 0) ws.mt[i] = msgs[f.a_idx * VEC + j];
+    ws.mb[i] = msgs[f.b_idx * VEC + j];
+  }
+  k.ids = 0;
+  if (lane < 18) {
+    const int t = lane / 3, u = lane - 3 * t;
+    int i, j;
+    f.node(t, 2 * u + ((((t & 1) != 0) != k.chk0) ? 1 : 0), &i, &j);
+    const int fr = c.frame[i * c.g.W + j];
+    const bool alpha_is_z = ((i & 1) == 0) == (f.dir == kDirR || f.dir == kDirL);
+    k.ids = alpha_is_z ? fr : (((fr & 1) << 1) | (fr >> 1));
+  }
+  k.A = ws.s0; k.B = ws.s1; k.mt = ws.mt; k.mb = ws.mb;
+  k.in = f.in_idx >= 0 ? msgs + f.in_idx * VEC : nullptr;
+  k.pI = c.pI; k.pE = c.pE;
+  k.a = f.a_idx >= 0;
+  k.lane = lane;
+  __syncwarp();
+  if (k.chk0) k.run_c();
+  else k.run_q();
+}
+
 // Block sides up to 4: one out-of-line copy (the kernels that also hold the
 // register forms keep their hot loop small in the instruction cache);
 // block sides 5 and 6 inline it (their loop is this sweep).
@@ -870,8 +917,8 @@ template <> __device__ __forceinline__ double pow2_neg<double>(int e) {
 
 // Resident CTAs per SM the register budget is sized for: 16 warps per SM in
 // FP32 and 8 in FP64; with k = 6 states (16 KB a buffer in FP32) the shared
-// memory decides.  LB > 0: the register-form-only kernel, sized for LB
-// resident CTAs per SM.
+// memory decides.  LB > 0: the kernel with small per-warp buffers
+// (fused_slot), sized for LB resident CTAs per SM.
 template <typename T, int NW, int G, int K, int LB = 0> struct FusedMinBlocks {
   static constexpr int warps = K > 4 ? NW : (sizeof(T) == 4 ? 16 : 8);
   static constexpr int value = LB > 0 ? LB : (warps / NW > 1 ? warps / NW : 1);
@@ -880,7 +927,7 @@ template <typename T, int NW, int G, int K, int LB = 0> struct FusedMinBlocks {
 // Position lists of a CTA: each colour's messages grouped by class, the
 // register forms first (class 2 shape + srev, so that a pass rarely mixes
 // both orders of the side messages), the node-by-node path last.
-constexpr int kClasses = 9;                 // per colour: 4 shapes x 2 orders, then none
+constexpr int kClasses = 10;                // per colour: 4 shapes x 2 orders, then none (R and D, L and U)
 template <int V> struct IntC { static constexpr int value = V; };
 
 // Cosets c0 .. c0 + G - 1 of one syndrome decoded by the whole CTA: syn_src
@@ -894,9 +941,9 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   const int W = g.W, d = g.d, nb = g.nb, WW = W * W;
   static_assert(K <= 4 || G == 1, "k = 6 states hold one coset per CTA");
   constexpr int VEC = FusedDim<K>::vec;
-  constexpr bool kLean = LB > 0;
-  static_assert(!kLean || K == 4, "register-form-only kernels are for k = 4");
-  const FusedLayout Lo = fused_layout<T, K>(g, M, NW, G, GM, kLean);
+  constexpr bool kLean = LB > 0 && K == 4;   // every block update in register form
+  static_assert(LB == 0 || K != 4 || !GM, "register-form-only kernels keep their messages in shared memory");
+  const FusedLayout Lo = fused_layout<T, K>(g, M, NW, G, GM, LB > 0);
   unsigned long long* px = reinterpret_cast<unsigned long long*>(smem + Lo.parity);
   unsigned long long* pz = px + d;
   uint8_t* frames = smem + Lo.frame;
@@ -910,13 +957,13 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   double* rlog = reinterpret_cast<double*>(smem + Lo.rlog);
   // misc: [0], [1] work counters of the two colours' node-by-node messages,
   // [2] the read-out's, [3] cosets converged (bit q), [4 + q] flags, [8 + q]
-  // iterations done, [12 .. 29] messages per (colour, class), [30 .. 47]
+  // iterations done, [12 .. 31] messages per (colour, class), [32 .. 51]
   // their list positions; dsh[q]: the sum of coset q's Delta terms at its
   // last iteration.
   int* misc = reinterpret_cast<int*>(smem + Lo.misc);
   double* dsh = reinterpret_cast<double*>(smem + Lo.misc + 208);
   int* cls_n = misc + 12;
-  int* cls_at = misc + 30;
+  int* cls_at = misc + 12 + 2 * kClasses;
   T* msgs = GM ? gmsgs : reinterpret_cast<T*>(smem + Lo.msgs);
   const int stride = fused_coset_stride<K>(M, GM);           // from one coset's messages to the next
 
@@ -952,13 +999,13 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
     if (d > 33) b1 = __ballot_sync(kFull, lane + 32 < d - 1 && src[(lane + 32) * step]);
     if (lane == 0) px[r] = prefix_parity(b0 | ((unsigned long long)b1 << 32));   // pz follows px
   }
-  if (tid < 48) misc[tid] = 0;
+  if (tid < 52) misc[tid] = 0;
   if (tid < 4) dsh[tid] = 0.0;
   __syncthreads();
   // Message table in (I, J, dir) order, and each message's rank in its class.
   const int NK = nb * nb * 4;
   auto class_of = [&](int I, int J, int dir) {
-    int c = 8;
+    int c = 8 + (dir & 1);                   // one direction's code at a time: k = 6 blocks have two forms
     if (reg) {
       const RegFrame f = reg_frame(g, I, J, dir);
       const int sh = f.shape();
@@ -1088,7 +1135,7 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   c.frame = frames; c.msg_of = msg_of; c.msg_off = nullptr; c.dims = nullptr;
   c.arena = nullptr; c.e0 = nullptr; c.cta_flags = &misc[4];
   FusedWS<T> ws{};
-  if constexpr (!kLean) ws = fused_ws_at<T, K>(smem + Lo.ws + warp * Lo.ws_stride, G);
+  if constexpr (!kLean) ws = fused_ws_at<T, K>(smem + Lo.ws + warp * Lo.ws_stride, G, fused_slot<K>(g, LB > 0));
 
   const T pI = a.pI_w, pE = a.pE_w;
   RegUpd<T> upd{a.eta_w, a.one_m_eta_w, T(0), T(0), ovl, M};
@@ -1121,7 +1168,7 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
       }
       // The node-by-node path: whole messages, every coset at once.
       if constexpr (!kLean) {
-        const int cnt = cls_n[color * kClasses + 8], at = cls_at[color * kClasses + 8];
+        const int cnt = cls_n[color * kClasses + 8] + cls_n[color * kClasses + 9], at = cls_at[color * kClasses + 8];
         c.frame = frames + (cos_of & 3u) * WW;
         if (tid == 0) misc[color ^ 1] = 0;           // the other colour's counter, idle until the barrier
         for (;;) {
@@ -1133,7 +1180,8 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
           if (!dev_check(idx >= 0 && idx < M, &misc[4])) continue;
           const int key = meta[idx];
           const Frame f = make_frame(c, key / 4 / nb, (key / 4) % nb, key & 3);
-          fused_sweep(ws, c, msgs, stride, cos_of, n, frames, f, (LogAcc<T>*)nullptr, lane);
+          if (K > 4 && f.h == 6 && f.ncols == 6) block6_update(ws, c, msgs, f, lane);
+          else fused_sweep(ws, c, msgs, stride, cos_of, n, frames, f, (LogAcc<T>*)nullptr, lane);
           fused_update<T, K>(ws, msgs, stride, cos_of, n, idx, f.h, upd.eta, upd.one_m_eta, ovl, M, lane);
         }
       }
@@ -1249,7 +1297,11 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   if constexpr (!kLean) {
     const unsigned all = G == 1 ? 0u : (G == 2 ? 0x4u : 0xE4u);    // slot q holds coset q
     c.frame = frames;
-    for (;;) {
+    const int full = fused_ws_bytes<T, K>(g, G, false);            // full-size state buffers
+    const int nro = K > 4 && LB > 0 ? imin(NW, NW * Lo.ws_stride / full) : NW;
+    if (K > 4 && LB > 0 && warp < nro)
+      ws = fused_ws_at<T, K>(smem + Lo.ws + warp * full, G, FusedDim<K>::slot);
+    while (warp < nro) {
       int item = 0;
       if (lane == 0) item = atomicAdd(&misc[2], 1);
       item = __shfl_sync(kFull, item, 0);

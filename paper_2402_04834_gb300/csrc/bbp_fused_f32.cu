@@ -5,6 +5,13 @@
 namespace bbp {
 
 cudaError_t launch_fused_f32(const LaunchArgs& a, int warps, int cosets, bool gm, int lean, cudaStream_t st) {
+  if (lean > 0 && a.geo.k > 4) {           // small state buffers, sized for `lean` CTAs per SM
+    switch (warps * 100 + cosets * 10 + lean) {
+      case 1611: return launch_fused_nw<float, 16, 1, 6, true, 1>(a, st);
+      case 812: return launch_fused_nw<float, 8, 1, 6, true, 2>(a, st);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   if (lean > 0) {                          // every block update in register form, sized for `lean` CTAs per SM
     switch (warps * 100 + cosets * 10 + lean) {
       case 1611: return launch_fused_nw<float, 16, 1, 4, false, 1>(a, st);

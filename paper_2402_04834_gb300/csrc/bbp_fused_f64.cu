@@ -5,6 +5,12 @@
 namespace bbp {
 
 cudaError_t launch_fused_f64(const LaunchArgs& a, int warps, int cosets, bool gm, int lean, cudaStream_t st) {
+  if (lean > 0 && a.geo.k > 4) {           // small state buffers, sized for `lean` CTAs per SM
+    switch (warps * 100 + cosets * 10 + lean) {
+      case 811: return launch_fused_nw<double, 8, 1, 6, true, 1>(a, st);
+      default: return cudaErrorInvalidValue;
+    }
+  }
   if (lean > 0) {                          // every block update in register form, sized for `lean` CTAs per SM
     switch (warps * 100 + cosets * 10 + lean) {
       case 1611: return launch_fused_nw<double, 16, 1, 4, false, 1>(a, st);
@@ -159,7 +165,29 @@ bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, in
 // syndromes: 12.2 ms, all others 12.3 to 13.1) but for the smallest codes
 // ((4, 4, 3) at d = 5: 2.20 ms against 3.01); one syndrome 709 us with (16, 1),
 // 1232 with (4, 2).
+// Block sides 5 and 6 (messages in workspace slots, one coset per CTA): the
+// kernels with small state buffers, 16 warps per SM (8 in FP64).
 bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, int* warps, int* cosets, int* lean) {
+  if (g.k > 4) {
+    auto fit6 = [&](int w) {
+      const int smem = precision == 0 ? fused_smem_for<double, 6>(g, M, w, 1, true, true)
+                                      : fused_smem_for<float, 6>(g, M, w, 1, true, true);
+      return smem > kMaxSmemBytes ? 0 : kSmemPerSm / (smem + kSmemReservedPerCta);
+    };
+    *cosets = 1;
+    if (precision == 0) {
+      if (fit6(8) < 1) return false;
+      *warps = 8; *lean = 1;
+      return true;
+    }
+    if (4 * B > sms && fit6(8) >= 2) {
+      *warps = 8; *lean = 2;
+      return true;
+    }
+    if (fit6(16) < 1) return false;
+    *warps = 16; *lean = 1;
+    return true;
+  }
   auto fit = [&](int w, int c) {
     const int smem = precision == 0 ? fused_smem_for<double, 4>(g, M, w, c, false, true)
                                     : fused_smem_for<float, 4>(g, M, w, c, false, true);

@@ -60,3 +60,17 @@ def test_default_kernel_of_every_size_gives_the_same_bits(d, B):
     b = pkg.decode(s, pkg.DecoderParams(**base, messages=1 if d <= 46 else 2))
     for key in ("logp", "delta", "iters", "flags", "decision"):
         assert torch.equal(a[key], b[key]), key
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("d,k,B", [(4, 6, 5), (7, 6, 60), (8, 6, 3), (9, 6, 60), (13, 6, 3), (13, 5, 60), (16, 6, 45)])
+def test_default_kernel_of_large_blocks_gives_the_same_bits(d, k, B):
+    # Side remainders 1, 3 and 5 (partial blocks of every width share the
+    # launch with full 6 x 6 blocks), one CTA of 16 warps and two of 8 per SM.
+    _, _, S = synth.sample_syndromes(9700 + d, 0, B, d, 0.11)
+    s = torch.from_numpy(S).cuda()
+    base = dict(d=d, k=k, p=0.11, max_iter=5, delta0=2e-3, precision="fp32", algorithm="fused")
+    a = pkg.decode(s, pkg.DecoderParams(**base))
+    b = pkg.decode(s, pkg.DecoderParams(**base, warps=4, cosets=1, messages=2))
+    for key in ("logp", "delta", "iters", "flags", "decision"):
+        assert torch.equal(a[key], b[key]), key
