@@ -22,7 +22,7 @@ BUILD_CHECKS = os.path.join(HERE, "_build_checks")
 LIB_CHECKS = os.path.join(HERE, "libblockbp_checks.so")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 SOURCES = ["bbp_api.cu", "bbp_decode_f64.cu", "bbp_decode_f32.cu", "bbp_fused_f32.cu", "bbp_fused_f64.cu",
-           "bbp_fused_mixed_f32.cu",
+           "bbp_fused_mixed_f32.cu", "bbp_fused_any_f32.cu", "bbp_fused_any_f64.cu",
            "bbp_sample.cu", "bbp_static.cu", "bbp_warm.cu", "bbp_warm_tc.cu",
            "bbp_warm_train.cu", "bbp_warm_decode.cu"]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

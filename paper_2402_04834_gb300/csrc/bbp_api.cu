@@ -29,19 +29,19 @@ bool shape_of(const bbp_params* p, const Geo& g, int M, int* warps, int* cosets,
 }
 
 // A launch that asks for no shape takes the kernel measured fastest for its
-// geometry and batch.  lean_ok: every syndrome is known to have odd distance;
+// geometry and batch.  odd: every syndrome is known to have odd distance;
 // mixed: smaller distances share the launch, so kernels whose buffers depend
 // on more than the largest one's size (k = 5, 6) are left out.
 void pick_default(const bbp_params* p, const Geo& g, int M, int64_t B, int* warps, int* cosets, bool* gm, int* lean,
-                  bool lean_ok, bool mixed) {
+                  bool odd, bool mixed) {
   if (p->launch_warps != 0 || p->launch_cosets != 0 || (p->launch_messages != 0 && p->launch_messages != (g.k > 4 ? 2 : 3)))
     return;
-  if (g.k < 4 || (g.k == 4 && (!lean_ok || g.d % 2 == 0)) || (g.k > 4 && mixed)) return;
+  if (g.k < 4 || (g.k > 4 && mixed)) return;
   int dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess ||
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
     return;
-  if (bbp::fused_pick(p->precision, g, M, B, sms, warps, cosets, lean)) *gm = g.k > 4;
+  if (bbp::fused_pick(p->precision, g, M, B, sms, odd, warps, cosets, lean)) *gm = g.k > 4;
 }
 
 int check_params(const bbp_params* p) {
@@ -189,9 +189,13 @@ int bbp_decode_batch_ex(const uint8_t* syndromes, int64_t B, const bbp_params* p
     if (s.warps == 0) return BBP_EUNSUPPORTED;
     int warps = s.warps, cosets = s.cosets, lean = s.lean;
     bool gm = s.gm;
-    pick_default(prm, s.g, s.M, B, &warps, &cosets, &gm, &lean, true, false);
-    e = prm->precision == BBP_FP64 ? bbp::launch_fused_f64(a, warps, cosets, gm, lean, st)
-                                   : bbp::launch_fused_f32(a, warps, cosets, gm, lean, st);
+    pick_default(prm, s.g, s.M, B, &warps, &cosets, &gm, &lean, prm->d % 2 != 0, false);
+    if (lean >= 10)
+      e = prm->precision == BBP_FP64 ? bbp::launch_fused_any_f64(a, warps, cosets, lean, st)
+                                     : bbp::launch_fused_any_f32(a, warps, cosets, lean, st);
+    else
+      e = prm->precision == BBP_FP64 ? bbp::launch_fused_f64(a, warps, cosets, gm, lean, st)
+                                     : bbp::launch_fused_f32(a, warps, cosets, gm, lean, st);
   } else
     e = prm->precision == BBP_FP64 ? bbp::launch_decode_f64(a, st) : bbp::launch_decode_f32(a, st);
   if (e != cudaSuccess) return BBP_ECUDA;
@@ -274,8 +278,13 @@ int bbp_decode_mixed(const uint8_t* syndromes, const int64_t* offsets, const int
     if (workspace_bytes < 256 + (size_t)m.slots * fused_slot_bytes(prm->k, c, Mmax, elem)) return BBP_ENOSPACE;
     m.slot_base = static_cast<char*>(workspace) + 256;
   }
-  cudaError_t e = prm->precision == BBP_FP64 ? bbp::launch_fused_mixed_f64(a, m, w, c, gm, lean, st)
-                                             : bbp::launch_fused_mixed_f32(a, m, w, c, gm, lean, st);
+  cudaError_t e;
+  if (lean >= 10)
+    e = prm->precision == BBP_FP64 ? bbp::launch_fused_mixed_any_f64(a, m, w, c, lean, st)
+                                   : bbp::launch_fused_mixed_any_f32(a, m, w, c, lean, st);
+  else
+    e = prm->precision == BBP_FP64 ? bbp::launch_fused_mixed_f64(a, m, w, c, gm, lean, st)
+                                   : bbp::launch_fused_mixed_f32(a, m, w, c, gm, lean, st);
   if (e != cudaSuccess) return BBP_ECUDA;
   e = bbp::launch_decide(a, st);
   return e == cudaSuccess ? BBP_OK : BBP_ECUDA;

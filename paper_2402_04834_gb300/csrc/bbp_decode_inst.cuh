@@ -57,7 +57,7 @@ cudaError_t launch_decode_t(const LaunchArgs& a, cudaStream_t st) {
 }
 
 template <typename T, int K>
-int fused_smem_for(const Geo& g, int M, int warps, int cosets, bool gm = (K > 4), bool lean = false) {
+int fused_smem_for(const Geo& g, int M, int warps, int cosets, bool gm = (K > 4), int lean = 0) {
   return fused_layout<T, K>(g, M, warps, cosets, gm, lean).total;
 }
 
@@ -100,7 +100,7 @@ cudaError_t persistent_grid(Kern kern, int threads, int smem, int ctas_per_sm, l
 template <typename T, int NW, int G, int K, bool GM = (K > 4), int LB = 0>
 cudaError_t launch_fused_nw(const LaunchArgs& a, cudaStream_t st) {
   const KArgs<T> k = fused_args<T>(a);
-  const int smem = fused_smem_for<T, K>(a.geo, a.M, NW, G, GM, LB > 0);
+  const int smem = fused_smem_for<T, K>(a.geo, a.M, NW, G, GM, LB == 0 ? 0 : (K == 4 && LB >= kEvenLB ? 2 : 1));
   auto kern = fused_kernel<T, NW, G, K, GM, LB>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
@@ -125,7 +125,7 @@ cudaError_t launch_fused_mixed_nw(const LaunchArgs& a, const MixedLaunch& m, cud
   const Geo gmax = make_geo(m.d_max, a.geo.k);
   int Mmax = 0, ae = 0;
   count_messages(gmax, 1, &Mmax, &ae);
-  const int smem = fused_smem_for<T, K>(gmax, Mmax, NW, G, GM, LB > 0);
+  const int smem = fused_smem_for<T, K>(gmax, Mmax, NW, G, GM, LB == 0 ? 0 : (K == 4 && LB >= kEvenLB ? 2 : 1));
   auto kern = fused_mixed_kernel<T, NW, G, K, GM, LB>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;

@@ -64,13 +64,13 @@ struct FusedWS {   // (sizes for block side K: slot = FusedDim<K>::slot, vec = F
 // full blocks node by node, takes full-size buffers from the same memory with
 // fewer warps.
 template <int K>
-BBP_HD int fused_slot(const Geo& g, bool lean) {
+BBP_HD int fused_slot(const Geo& g, int lean) {
   if (K <= 4 || !lean) return FusedDim<K>::slot;
   return g.k == 6 && g.W % 6 == 5 ? 2 * kBlock6Buf : kBlock6Buf;   // a 6 x 5 block's widest state has 2^11 entries
 }
 
 template <typename T, int K>
-BBP_HD int fused_ws_bytes(const Geo& g, int G, bool lean = false) {
+BBP_HD int fused_ws_bytes(const Geo& g, int G, int lean = 0) {
   if (K == 4 && lean) return align_up((int)sizeof(T) * kRegStage, 16);
   return align_up((int)sizeof(T) * G * (2 * fused_slot<K>(g, lean) + 16 + 2 * FusedDim<K>::vec), 16);
 }
@@ -107,19 +107,25 @@ struct FusedLayout {
 };
 
 // gm: the messages live in a workspace slot of the CTA (always for k = 5,
-// 6; on request for k <= 4), not in shared memory.
+// 6; on request for k <= 4), not in shared memory.  lean: the kernels with
+// small per-warp buffers; at k = 4, 1 where every block is four or one node
+// wide, 2 where any distance may come: blocks three nodes wide are then read
+// out node by node by kReadWarps warps, a coset at a time, in the buffers'
+// place.
+constexpr int kReadWarps = 4;
+constexpr int kEvenLB = 10;                 // template argument LB of the kernels with lean = 2: kEvenLB + CTAs per SM
 template <typename T, int K>
-BBP_HD FusedLayout fused_layout(const Geo& g, int M, int nwarps, int G, bool gm = (K > 4), bool lean = false) {
+BBP_HD FusedLayout fused_layout(const Geo& g, int M, int nwarps, int G, bool gm = (K > 4), int lean = 0) {
   FusedLayout L;
   int o = 0;
   L.parity = o; o = align_up(o + 2 * g.d * 8, 16);             // the pure error, as prefix parities
-  L.frame = o;  if (!lean || K > 4) o = align_up(o + G * g.W * g.W, 16);
-  L.msg_of = o; if (!lean || K > 4) o = align_up(o + 2 * g.nb * g.nb * 4, 16);
+  L.frame = o;  if (lean != 1 || K > 4) o = align_up(o + G * g.W * g.W, 16);
+  L.msg_of = o; if (lean != 1 || K > 4) o = align_up(o + 2 * g.nb * g.nb * 4, 16);
   L.meta = o;   o = align_up(o + 2 * M, 16);
   L.work = o;   o = align_up(o + 2 * M, 16);                   // lists of both colours
   L.ovl = o;    o = align_up(o + (int)sizeof(T) * G * M, 16);
   L.rlog = o;   o = align_up(o + 8 * G * (g.nb * g.nb + M / 2), 16);
-  L.misc = o;   o = align_up(o + 256, 16);
+  L.misc = o;   o = align_up(o + 336, 16);
   // Register form (k = 4): a task per message and the qubit ids of each
   // (coset, message), by list position, built once per syndrome.
   L.tasks = o;  if (K == 4 && g.k == 4) o = align_up(o + (int)sizeof(RegTask) * M, 16);
@@ -129,7 +135,9 @@ BBP_HD FusedLayout fused_layout(const Geo& g, int M, int nwarps, int G, bool gm 
   if (!gm) o = align_up(o + (int)sizeof(T) * G * fused_coset_stride<K>(M, gm), 16);
   L.ws = o;
   L.ws_stride = fused_ws_bytes<T, K>(g, G, lean);
-  o = align_up(o + nwarps * L.ws_stride, 16);
+  int ws = nwarps * L.ws_stride;
+  if (K == 4 && lean == 2) ws = imax(ws, kReadWarps * fused_ws_bytes<T, K>(g, 1));
+  o = align_up(o + ws, 16);
   L.total = o;
   return L;
 }
@@ -921,13 +929,14 @@ template <> __device__ __forceinline__ double pow2_neg<double>(int e) {
 // (fused_slot), sized for LB resident CTAs per SM.
 template <typename T, int NW, int G, int K, int LB = 0> struct FusedMinBlocks {
   static constexpr int warps = K > 4 ? NW : (sizeof(T) == 4 ? 16 : 8);
-  static constexpr int value = LB > 0 ? LB : (warps / NW > 1 ? warps / NW : 1);
+  static constexpr int value = LB > 0 ? LB % kEvenLB : (warps / NW > 1 ? warps / NW : 1);
 };
 
 // Position lists of a CTA: each colour's messages grouped by class, the
 // register forms first (class 2 shape + srev, so that a pass rarely mixes
 // both orders of the side messages), the node-by-node path last.
-constexpr int kClasses = 10;                // per colour: 4 shapes x 2 orders, then none (R and D, L and U)
+constexpr int kClassNone = 2 * kShapes;
+constexpr int kClasses = kClassNone + 2;    // per colour: shapes x 2 orders, then none (R and D, L and U)
 template <int V> struct IntC { static constexpr int value = V; };
 
 // Cosets c0 .. c0 + G - 1 of one syndrome decoded by the whole CTA: syn_src
@@ -942,8 +951,10 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   static_assert(K <= 4 || G == 1, "k = 6 states hold one coset per CTA");
   constexpr int VEC = FusedDim<K>::vec;
   constexpr bool kLean = LB > 0 && K == 4;   // every block update in register form
+  constexpr bool kEven = kLean && LB >= kEvenLB;   // ... blocks three nodes wide included
+  constexpr int kMode = LB == 0 ? 0 : (kEven ? 2 : 1);
   static_assert(LB == 0 || K != 4 || !GM, "register-form-only kernels keep their messages in shared memory");
-  const FusedLayout Lo = fused_layout<T, K>(g, M, NW, G, GM, LB > 0);
+  const FusedLayout Lo = fused_layout<T, K>(g, M, NW, G, GM, kMode);
   unsigned long long* px = reinterpret_cast<unsigned long long*>(smem + Lo.parity);
   unsigned long long* pz = px + d;
   uint8_t* frames = smem + Lo.frame;
@@ -957,18 +968,18 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   double* rlog = reinterpret_cast<double*>(smem + Lo.rlog);
   // misc: [0], [1] work counters of the two colours' node-by-node messages,
   // [2] the read-out's, [3] cosets converged (bit q), [4 + q] flags, [8 + q]
-  // iterations done, [12 .. 31] messages per (colour, class), [32 .. 51]
+  // iterations done, [12 .. 43] messages per (colour, class), [44 .. 75]
   // their list positions; dsh[q]: the sum of coset q's Delta terms at its
   // last iteration.
   int* misc = reinterpret_cast<int*>(smem + Lo.misc);
-  double* dsh = reinterpret_cast<double*>(smem + Lo.misc + 208);
+  double* dsh = reinterpret_cast<double*>(smem + Lo.misc + 304);
   int* cls_n = misc + 12;
   int* cls_at = misc + 12 + 2 * kClasses;
   T* msgs = GM ? gmsgs : reinterpret_cast<T*>(smem + Lo.msgs);
   const int stride = fused_coset_stride<K>(M, GM);           // from one coset's messages to the next
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if constexpr (kLean) {
+  if constexpr (kLean && !kEven) {
     // The host launches register-form-only kernels only where every block has
     // a register form; in a mixed batch the caller vouches for it.
     if (!register_form_only(g)) {
@@ -999,13 +1010,13 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
     if (d > 33) b1 = __ballot_sync(kFull, lane + 32 < d - 1 && src[(lane + 32) * step]);
     if (lane == 0) px[r] = prefix_parity(b0 | ((unsigned long long)b1 << 32));   // pz follows px
   }
-  if (tid < 52) misc[tid] = 0;
+  if (tid < 76) misc[tid] = 0;
   if (tid < 4) dsh[tid] = 0.0;
   __syncthreads();
   // Message table in (I, J, dir) order, and each message's rank in its class.
   const int NK = nb * nb * 4;
   auto class_of = [&](int I, int J, int dir) {
-    int c = 8 + (dir & 1);                   // one direction's code at a time: k = 6 blocks have two forms
+    int c = kClassNone + (dir & 1);                   // one direction's code at a time: k = 6 blocks have two forms
     if (reg) {
       const RegFrame f = reg_frame(g, I, J, dir);
       const int sh = f.shape();
@@ -1022,13 +1033,13 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
         meta[idx] = (int16_t)key;
         rank[idx] = (int16_t)atomicAdd(&cls_n[class_of(I, J, dir)], 1);
       }
-      if constexpr (!kLean) msg_of[key] = (int16_t)idx;
+      if constexpr (!kLean || kEven) msg_of[key] = (int16_t)idx;
     } else {
-      if constexpr (!kLean) msg_of[key] = -1;
+      if constexpr (!kLean || kEven) msg_of[key] = -1;
     }
   }
   // Every coset's frame, for the node-by-node path.
-  if constexpr (!kLean) {
+  if constexpr (!kLean || kEven) {
     for (int e = tid; e < G * WW; e += NW * 32) {
       const int q = e / WW, ij = e - q * WW;
       const int i = ij / W, j = ij - i * W;
@@ -1064,7 +1075,7 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
     const int pos = cls_at[cls] + rank[idx];
     if (!dev_check(pos >= 0 && pos < M, &misc[4])) continue;
     work[pos] = (int16_t)idx;
-    if (cls % kClasses < 8) {
+    if (cls % kClasses < kClassNone) {
       const RegFrame f = reg_frame(g, I, J, dir);
       RegTask q = reg_task(g, M, I, J, f);
       if (!dev_check((q.in & kTaskIdx) < M + kBorderVecs && (q.up & kTaskIdx) < M + kBorderVecs &&
@@ -1135,14 +1146,10 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   c.frame = frames; c.msg_of = msg_of; c.msg_off = nullptr; c.dims = nullptr;
   c.arena = nullptr; c.e0 = nullptr; c.cta_flags = &misc[4];
   FusedWS<T> ws{};
-  if constexpr (!kLean) ws = fused_ws_at<T, K>(smem + Lo.ws + warp * Lo.ws_stride, G, fused_slot<K>(g, LB > 0));
+  if constexpr (!kLean) ws = fused_ws_at<T, K>(smem + Lo.ws + warp * Lo.ws_stride, G, fused_slot<K>(g, kMode));
 
   const T pI = a.pI_w, pE = a.pE_w;
-  RegUpd<T> upd{a.eta_w, a.one_m_eta_w, T(0), T(0), ovl, M};
-  if constexpr (sizeof(T) == 8) {
-    upd.rho = pI / pE;
-    upd.rho_m1 = (pI - pE) / pE;
-  }
+  const RegUpd<T> upd{a.eta_w, a.one_m_eta_w, ovl, M};
   unsigned act = (1u << G) - 1;                      // cosets still iterating
   for (int it = 1; it <= a.max_iter && M > 0 && act; ++it) {
     int n = 0;
@@ -1162,13 +1169,22 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
                                                      n, first, warp, lane, upd);
           first += reg_updates<T, GM, kShapeCol, NW>(stage, pI, pE, ms, tasks, qid, M, ca[2], cn[2] + cn[3], cos_of,
                                                      n, first, warp, lane, upd);
-          reg_updates<T, GM, kShapeDot, NW>(stage, pI, pE, ms, tasks, qid, M, ca[6], cn[6] + cn[7], cos_of, n, first,
-                                            warp, lane, upd);
+          first += reg_updates<T, GM, kShapeDot, NW>(stage, pI, pE, ms, tasks, qid, M, ca[6], cn[6] + cn[7], cos_of, n,
+                                                     first, warp, lane, upd);
+          if constexpr (!kLean || kEven) {
+            first += reg_updates<T, GM, kShape34, NW>(stage, pI, pE, ms, tasks, qid, M, ca[10], cn[10] + cn[11], cos_of,
+                                                      n, first, warp, lane, upd);
+            first += reg_updates<T, GM, kShape43, NW>(stage, pI, pE, ms, tasks, qid, M, ca[8], cn[8] + cn[9], cos_of, n,
+                                                      first, warp, lane, upd);
+            reg_updates<T, GM, kShape33, NW>(stage, pI, pE, ms, tasks, qid, M, ca[12], cn[12] + cn[13], cos_of, n, first,
+                                             warp, lane, upd);
+          }
         }
       }
       // The node-by-node path: whole messages, every coset at once.
       if constexpr (!kLean) {
-        const int cnt = cls_n[color * kClasses + 8] + cls_n[color * kClasses + 9], at = cls_at[color * kClasses + 8];
+        const int cnt = cls_n[color * kClasses + kClassNone] + cls_n[color * kClasses + kClassNone + 1];
+        const int at = cls_at[color * kClasses + kClassNone];
         c.frame = frames + (cos_of & 3u) * WW;
         if (tid == 0) misc[color ^ 1] = 0;           // the other colour's counter, idle until the barrier
         for (;;) {
@@ -1227,6 +1243,19 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
       rlog[q * per + at] = at < nblk ? log(fabs(v)) : -log(fabs(v));
     }
     if (!(v > T(0))) atomicOr(&misc[4 + q], at < nblk ? kFlagBlock : kFlagOverlap);
+  };
+  // A block contracted node by node: its norms taken out on the way and z.
+  auto close_block = [&](LogAcc<T>& l, T z, int q, int at) {
+    if (lane == 0) {
+      l.mul(z < T(0) ? -z : z);
+      if constexpr (sizeof(T) == 4) {
+        reinterpret_cast<float*>(rlog + q * per + at)[0] = l.m;
+        reinterpret_cast<int*>(rlog + q * per + at)[1] = l.e;
+      } else {
+        rlog[q * per + at] = l.value();
+      }
+      if (!(z > T(0))) atomicOr(&misc[4 + q], kFlagBlock);
+    }
   };
   int first = 0;                                     // passes dealt to the warps so far
   if constexpr (K == 4) {
@@ -1294,10 +1323,31 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
       blocks(IntC<kShapeDot>{}, edge ? 1 : 0, [&](int i, int& I, int& J) { I = J = nf; });
     }
   }
+  if constexpr (kEven) {
+    // Node by node: the blocks three nodes wide, a coset at a time; no other
+    // warp's buffers are in use any more but the passes' above.
+    const int nf = W / 4, cnt = W % 4 == 3 ? 2 * nf + 1 : 0;
+    __syncthreads();
+    ws = fused_ws_at<T, K>(smem + Lo.ws + (warp < kReadWarps ? warp : 0) * fused_ws_bytes<T, K>(g, 1), 1,
+                           FusedDim<K>::slot);
+    for (int j = warp; warp < kReadWarps && j < cnt * G; j += kReadWarps) {
+      const int i = j / G, q = j % G;
+      const int I = i < nf ? i : nf, J = i < nf ? nf : i - nf;     // (i, nf), (nf, 0 .. nf)
+      c.frame = frames + q * WW;
+      const Frame f = make_frame(c, I, J, kDirR);
+      LogAcc<T> ls[kFusedMaxG];
+      fused_sweep(ws, c, msgs, stride, (unsigned)q, 1, frames, f, ls, lane);
+      const int right = J + 1 < nb ? msg_index(c, I, J + 1, kDirL) : -1;
+      if (!dev_check(right >= -1 && right < M, &misc[4])) continue;
+      close_block(ls[0], right >= 0 ? read_dot(ws.s0, msgs + q * stride + right * VEC, 1 << f.h, lane) : ws.s0[0], q,
+                  I * nb + J);
+      __syncwarp();
+    }
+  }
   if constexpr (!kLean) {
     const unsigned all = G == 1 ? 0u : (G == 2 ? 0x4u : 0xE4u);    // slot q holds coset q
     c.frame = frames;
-    const int full = fused_ws_bytes<T, K>(g, G, false);            // full-size state buffers
+    const int full = fused_ws_bytes<T, K>(g, G);                   // full-size state buffers
     const int nro = K > 4 && LB > 0 ? imin(NW, NW * Lo.ws_stride / full) : NW;
     if (K > 4 && LB > 0 && warp < nro)
       ws = fused_ws_at<T, K>(smem + Lo.ws + warp * full, G, FusedDim<K>::slot);
@@ -1307,7 +1357,8 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
       item = __shfl_sync(kFull, item, 0);
       if (item >= nblk) break;
       const int I = item / nb, J = item % nb;
-      if (reg && reg_frame(g, I, J, kDirR).shape() != kShapeNone) continue;
+      const int shape = reg_frame(g, I, J, kDirR).shape();
+      if (reg && shape != kShapeNone && shape <= kShapeDot) continue;   // read out above
       const Frame f = make_frame(c, I, J, kDirR);
       LogAcc<T> ls[kFusedMaxG];
       fused_sweep(ws, c, msgs, stride, all, G, frames, f, ls, lane);
@@ -1319,16 +1370,7 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
         // carry the value 0, so only entry 0 survives.
         const T z = right >= 0 ? read_dot(ws.s0 + (q << f.h), msgs + q * stride + right * VEC, 1 << f.h, lane)
                                : ws.s0[q << f.h];
-        if (lane == 0) {
-          ls[q].mul(z < T(0) ? -z : z);
-          if constexpr (sizeof(T) == 4) {
-            reinterpret_cast<float*>(rlog + q * per + item)[0] = ls[q].m;
-            reinterpret_cast<int*>(rlog + q * per + item)[1] = ls[q].e;
-          } else {
-            rlog[q * per + item] = ls[q].value();
-          }
-          if (!(z > T(0))) atomicOr(&misc[4 + q], kFlagBlock);
-        }
+        close_block(ls[q], z, q, item);
       }
       __syncwarp();
     }

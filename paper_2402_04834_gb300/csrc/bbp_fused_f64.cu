@@ -160,14 +160,16 @@ bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, in
 // half-round for 8 warps: four warps where six such CTAs fit (d <= 9; d = 5,
 // 10^4 syndromes 1.58 ms against 1.78), or five and the batch is long enough
 // to hide its slower CTAs' tail (d = 11, 10^4 syndromes 4.93 ms against 5.06).
-// Where four cosets do not fit (d >= 27), two or one.  FP64 is bound by its
-// pipe, so at large batches the shape matters little ((8, 2, 2) at d = 11, 1000
-// syndromes: 12.2 ms, all others 12.3 to 13.1) but for the smallest codes
-// ((4, 4, 3) at d = 5: 2.20 ms against 3.01); one syndrome 709 us with (16, 1),
-// 1232 with (4, 2).
+// Where four cosets do not fit (d >= 27), two or one.  Batches that may hold
+// even distances take the kernels that know three-wide blocks too, by the
+// same rule.  FP64 is bound by its pipe, so at large batches the shape
+// matters little (within 7 % at d = 11, 1000 syndromes) but for the smallest
+// codes ((4, 4, 3) at d = 5, 1000 syndromes: a quarter less than (8, 2, 2));
+// small batches gain most (one syndrome at d = 11: (16, 1) 0.58 of (4, 2)).
 // Block sides 5 and 6 (messages in workspace slots, one coset per CTA): the
 // kernels with small state buffers, 16 warps per SM (8 in FP64).
-bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, int* warps, int* cosets, int* lean) {
+bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, bool odd, int* warps, int* cosets,
+                int* lean) {
   if (g.k > 4) {
     auto fit6 = [&](int w) {
       const int smem = precision == 0 ? fused_smem_for<double, 6>(g, M, w, 1, true, true)
@@ -189,23 +191,23 @@ bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, int* w
     return true;
   }
   auto fit = [&](int w, int c) {
-    const int smem = precision == 0 ? fused_smem_for<double, 4>(g, M, w, c, false, true)
-                                    : fused_smem_for<float, 4>(g, M, w, c, false, true);
+    const int smem = precision == 0 ? fused_smem_for<double, 4>(g, M, w, c, false, odd ? 1 : 2)
+                                    : fused_smem_for<float, 4>(g, M, w, c, false, odd ? 1 : 2);
     return smem > kMaxSmemBytes ? 0 : kSmemPerSm / (smem + kSmemReservedPerCta);
   };
-  auto take = [&](int w, int c, int l) { *warps = w; *cosets = c; *lean = l; return true; };
+  auto take = [&](int w, int c, int l) { *warps = w; *cosets = c; *lean = odd ? l : kEvenLB + l; return true; };
   int c = 4 * B <= sms ? 1 : (2 * B <= sms ? 2 : 4);
   while (c > 1 && fit(16, c) < 1) c /= 2;
   if (fit(16, c) < 1) return false;
   if (precision == 0) {
     if (c < 4) return take(16, c, 1);
     if (B <= sms) return take(8, 4, 1);
-    if (fit(4, 4) >= 6) return take(4, 4, 3);
+    if (odd && fit(4, 4) >= 6) return take(4, 4, 3);
     return fit(8, 2) >= 2 ? take(8, 2, 2) : take(16, 2, 1);
   }
   if (B <= sms || c < 4 || fit(8, 4) < 2) return take(16, c, 1);
   if (B <= 2ll * sms) return take(8, 4, 2);
-  if (fit(4, 4) >= 6 || (fit(4, 4) >= 5 && B >= 16ll * sms)) return take(4, 4, 6);
+  if (odd && (fit(4, 4) >= 6 || (fit(4, 4) >= 5 && B >= 16ll * sms))) return take(4, 4, 6);
   const int n = fit(8, 4);
   return take(8, 4, n < 4 ? n : 4);
 }

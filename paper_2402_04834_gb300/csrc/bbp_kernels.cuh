@@ -76,25 +76,24 @@ __device__ __forceinline__ T group_sum(T v, int G) {
 
 // 1 / sqrt(s), 0 for s = 0: the scale of a unit-norm vector (Remark 3).
 // FP32 takes the hardware reciprocal square root (a scale factor, whose last
-// bit does not matter).  FP64 refines it by one third-order Newton (Halley)
-// step y + y r (1/2 + 3 r / 8), r = 1 - m y^2, which squares and more the
-// seed's 2^-22: five FP64 operations, where the rounded square root and
-// quotient were most of an update's (FP64 issues two lanes a cycle per SM).
-// The seed is taken of s scaled by an even power of two into [1, 4).
+// bit does not matter); FP64 the rounded square root and quotient.
 __device__ __forceinline__ float inv_norm(float s) { return s > 0.f ? rsqrtf(s) : 0.f; }
-// Reciprocal square root of m in [1, 4).
-__device__ __forceinline__ double rsqrt_unit(double m) {
+__device__ __forceinline__ double inv_norm(double s) { return s > 0.0 ? 1.0 / sqrt(s) : 0.0; }
+
+// The same within an ulp, in five FP64 operations, for the MPS form's linear
+// algebra (FP64 issues two lanes a cycle per SM): the FP32 seed y refined by
+// one third-order Newton (Halley) step y + y r (1/2 + 3 r / 8), r = 1 - m y^2.
+__device__ __forceinline__ double rsqrt_unit(double m) {   // m in [1, 4)
   const double y = (double)rsqrtf((float)m);
   const double r = fma(-(m * y), y, 1.0);
   return fma(y * r, fma(r, 0.375, 0.5), y);
 }
-__device__ __forceinline__ double inv_norm(double s) {
+__device__ __forceinline__ double inv_norm_ulp(double s) {
   if (!(s > 0.0)) return 0.0;
   const int hi = __double2hiint(s), e = hi >> 20;          // biased exponent (s > 0)
   if (e == 0 || e == 0x7ff) return 1.0 / sqrt(s);          // subnormal, infinity
-  const int k = (e - 1023) & ~1;
-  const double m = __hiloint2double(hi - (k << 20), __double2loint(s));
-  const double z = rsqrt_unit(m);
+  const int k = (e - 1023) & ~1;                           // s scaled by an even power of two into [1, 4)
+  const double z = rsqrt_unit(__hiloint2double(hi - (k << 20), __double2loint(s)));
   return __hiloint2double(__double2hiint(z) - ((k >> 1) << 20), __double2loint(z));
 }
 
@@ -582,7 +581,7 @@ __device__ __noinline__ void lq_step64(WarpWS<double, K, DM>& ws, int s, int lan
         continue;
       }
       if (pass == 0) kept |= 1u << j;
-      const double rs = inv_norm(nj2);
+      const double rs = inv_norm_ulp(nj2);
       const double lj = cf * rs;             // <x_row, q_j>; of row j its norm
       if (row == j) scale = rs;
       if (own && row >= j && half == 0) Lc[row * pl + j] = lj;
@@ -765,7 +764,7 @@ __device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<dou
   double* svt = ws.mat + 2 * DM * DM;        // r x n
   const FastDiv dn(n);
   if (on && rank < r) {
-    const double inv = tr ? 1.0 : inv_norm(sq);
+    const double inv = tr ? 1.0 : inv_norm_ulp(sq);
 #pragma unroll
     for (int t = 0; t < DM; ++t) {
       const int i = 2 * t + half;

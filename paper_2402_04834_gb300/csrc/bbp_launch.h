@@ -55,9 +55,10 @@ constexpr int kSmemReservedPerCta = 1024;       // reserved by the runtime per r
 bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, int* messages, bool allow_lean = true,
                  int* lean_blocks = nullptr);
 
-// The register-form-only kernel of a default launch (k = 4, odd d) for B
-// syndromes on sms SMs; false where the shape of fused_shape stands.
-bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, int* warps, int* cosets, int* lean);
+// The kernel of a default launch for B syndromes on sms SMs (k = 4: register
+// form only, odd: every distance is known to be odd; k = 5, 6: small state
+// buffers); false where the shape of fused_shape stands.
+bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, bool odd, int* warps, int* cosets, int* lean);
 
 struct MixedLaunch {
   const int32_t* d_of;
@@ -78,6 +79,13 @@ cudaError_t launch_fused_mixed_f64(const LaunchArgs& a, const MixedLaunch& mx, i
                                    int lean, cudaStream_t st);
 cudaError_t launch_fused_mixed_f32(const LaunchArgs& a, const MixedLaunch& mx, int warps, int cosets, bool gm,
                                    int lean, cudaStream_t st);
+// The register-form kernels for any distance (lean >= 10: 10 + CTAs per SM).
+cudaError_t launch_fused_any_f64(const LaunchArgs& a, int warps, int cosets, int lean, cudaStream_t st);
+cudaError_t launch_fused_any_f32(const LaunchArgs& a, int warps, int cosets, int lean, cudaStream_t st);
+cudaError_t launch_fused_mixed_any_f64(const LaunchArgs& a, const MixedLaunch& mx, int warps, int cosets, int lean,
+                                       cudaStream_t st);
+cudaError_t launch_fused_mixed_any_f32(const LaunchArgs& a, const MixedLaunch& mx, int warps, int cosets, int lean,
+                                       cudaStream_t st);
 cudaError_t launch_decode_f64(const LaunchArgs& a, cudaStream_t st);
 cudaError_t launch_decode_f32(const LaunchArgs& a, cudaStream_t st);
 cudaError_t launch_decide(const LaunchArgs& a, cudaStream_t st);

@@ -35,7 +35,10 @@ namespace bbp {
 
 constexpr int kRegVec = 16;                 // entries of a message vector
 constexpr int kBorderVecs = 2;              // product vectors of the grid border, after the messages
+// Shapes (chain height x columns): 4 x 4; 4 x 1, 1 x 4 and 1 x 1, the last
+// blocks of odd d; 4 x 3, 3 x 4 and 3 x 3, those of even d.
 constexpr int kShapeNone = 0, kShapeQuad = 1, kShapeCol = 2, kShapeRow = 3, kShapeDot = 4;
+constexpr int kShape43 = 5, kShape34 = 6, kShape33 = 7, kShapes = 7;
 
 // Index of the directed edge leaving block (I, J) towards dir in (I, J, dir)
 // order (R, L, D, U); the edge must exist.
@@ -85,12 +88,17 @@ struct RegFrame {
     node(0, 0, &i, &j);
     return (i + j) & 1;
   }
+  // Blocks three nodes wide or high keep the node-by-node form's chain order.
+  __device__ __forceinline__ bool wide3() const { return h == 3 || ncols == 3; }
   __device__ __forceinline__ bool srev() const { return dir == kDirL || dir == kDirU; }
   __device__ __forceinline__ int shape() const {
     if (h == 4 && ncols == 4) return kShapeQuad;
     if (h == 4 && ncols == 1) return kShapeCol;
     if (h == 1 && ncols == 4) return kShapeRow;
     if (h == 1 && ncols == 1) return kShapeDot;
+    if (h == 4 && ncols == 3) return kShape43;
+    if (h == 3 && ncols == 4) return kShape34;
+    if (h == 3 && ncols == 3) return kShape33;
     return kShapeNone;
   }
 };
@@ -107,7 +115,7 @@ __device__ __forceinline__ RegFrame reg_frame(const Geo& g, int I, int J, int di
 
 __device__ __forceinline__ RegTask reg_task(const Geo& g, int M, int I, int J, const RegFrame& f) {
   const int nb = g.nb;
-  const bool chk0 = f.chk0(), srev = f.srev(), rev = chk0 && f.h > 1;
+  const bool chk0 = f.chk0(), srev = f.srev(), rev = chk0 && f.h > 1 && !f.wide3();
   // The border vector of a side whose leg nearest the vector's last entry
   // belongs to node (i, j): mask bit 0 is set at a qubit.
   auto border = [&](int i, int j) { return M + (((i + j) & 1) ? 0 : 1); };
@@ -158,7 +166,8 @@ __device__ __forceinline__ int frame_bits(const unsigned long long* px, const un
 // and the bits that the logical strings X-bar (grid row 0) and Z-bar (column
 // 0) flip.  4 x 4: the upper (u = 0) and lower qubit of column t at bits
 // 2 (2 t + u); 4 x 1: the qubits at s' = 0 and 2; 1 x 4: the qubits of columns
-// 0 and 2, or 1 and 3; 1 x 1: the node.
+// 0 and 2, or 1 and 3; 1 x 1: the node; three wide or high: field 2 t + u the
+// qubit at chain position 2 u, or 2 u + 1 in a column that starts with a check.
 struct RegIds {
   unsigned id, fx, fz;
 };
@@ -197,6 +206,11 @@ __device__ __forceinline__ RegIds reg_ids(const RegFrame& f, const unsigned long
     add_id(v, f, chk0 ? 3 : 2, 0, 1, px, pz);
   } else if (shape == kShapeDot) {
     add_id(v, f, 0, 0, 0, px, pz);
+  } else if (shape != kShapeNone) {
+    for (int t = 0; t < f.ncols; ++t) {
+      const int c = ((t & 1) != 0) != chk0 ? 1 : 0;
+      for (int u = 0; 2 * u + c < f.h; ++u) add_id(v, f, t, 2 * u + c, 2 * t + u, px, pz);
+    }
   }
   return v;
 }
@@ -227,7 +241,6 @@ struct RegMsgs {
 template <typename T>
 struct RegUpd {
   T eta, one_m_eta;
-  T rho, rho_m1;                            // pi(I) / pi(X), that - 1 (FP64)
   T* ovl;                                   // Delta term of each (coset, message)
   int M;
 };
@@ -472,55 +485,56 @@ __device__ __forceinline__ void quad_pass(T* stage, T pI, T pE, const RegMsgs<T,
   // at once.  Column 2 (qubits at 0, 2) is the data column of both side
   // messages: the upper leg v is summed against A (above), the lower leg
   // w = r3 against B[b0 b1 w f].
-  T h0[2], h1[2], kk0[2], kk1[2];                          // by r0 ^ r2; by r2 ^ b1
+  T h0[2], h1[2];                                          // by r0 ^ r2
 #pragma unroll
   for (int b = 0; b < 2; ++b) {
     h0[b] = qco(tq, 2, (unsigned)b, pI, pE);
     h1[b] = qco(tq, 2, 2u + b, pI, pE);
-    kk0[b] = qco(tq, 3, (unsigned)b, pI, pE);
-    kk1[b] = qco(tq, 3, 2u + b, pI, pE);
   }
+  // Column 1's lower qubit scales T_b0 by g[b0 ^ r3][r2 ^ b1]: pE for the b0
+  // that its id does not meet (O), whatever b1, so S1, u and Y of that b0 are
+  // formed once for both b1; for the other b0 (h) pI where r2 ^ b1 meets the id.
+  const bool h = tq & 0x80u;
+  const T kh[2] = {(tq & 0x40u) ? pE : pI, (tq & 0x40u) ? pI : pE};   // by r2 ^ b1
+  const int lane_h = (lane & ~1) | (h ? 1 : 0), lane_o = lane_h ^ 1;
   const T c2k0 = qco(tq, 5, 0u, pI, pE), c2k1 = qco(tq, 5, 2u, pI, pE);
   // Column 3's upper leg e is tied to r0 by its check: only e = r0 of
   // A[a0 a1 v e] and of everything after it reaches a row's output.
-  T Y[2][2][2][2];                                         // [b0][b1][q0][q2], e = r0
+  T YO[2][2], Yh[2][2][2];                                 // [q0][q2], [b1][q0][q2], e = r0
 #pragma unroll
   for (int a0 = 0; a0 < 2; ++a0) {
     T cA[4];
     vcopy4(sj + 8 * r1 + 4 * a0, cA);                      // [alpha][q0]
-    T T0[2][2], T1[2][2];                                  // r3 = 0 and 1 of the upper qubit's butterfly over r1
+    T TO[2][2], Th[2][2];                                  // the upper qubit's butterfly over r1, r3 = !h and h
 #pragma unroll
     for (int a = 0; a < 2; ++a)
 #pragma unroll
       for (int b = 0; b < 2; ++b) {
         const T o = S0[a0][a][b];
         const T t = fma(h1[a ^ b], shx(o, 2), h0[a ^ b] * o);
-        T0[a][b] = __shfl_sync(kFull, t, lane & ~1);
-        T1[a][b] = __shfl_sync(kFull, t, lane | 1);
+        TO[a][b] = __shfl_sync(kFull, t, lane_o);
+        Th[a][b] = __shfl_sync(kFull, t, lane_h);
       }
 #pragma unroll
-    for (int b0 = 0; b0 < 2; ++b0)
+    for (int k = 0; k < 3; ++k) {                          // O, then h with b1 = 0, 1
+      T S1[2][2], u[2][2];
 #pragma unroll
-      for (int b1 = 0; b1 < 2; ++b1) {
-        T S1[2][2], u[2][2];
+      for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
+        for (int b = 0; b < 2; ++b) S1[a][b] = k == 0 ? pE * TO[a][b] : kh[(k - 1) ^ b] * Th[a][b];
 #pragma unroll
-          for (int b = 0; b < 2; ++b)
-            S1[a][b] = b0 == 0 ? kk0[b1 ^ b] * T0[a][b] : kk1[b1 ^ b] * T1[a][b];
+      for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
+        for (int b = 0; b < 2; ++b) u[a][b] = fma(c2k1, S1[a][b ^ 1], c2k0 * S1[a][b]);
 #pragma unroll
-          for (int b = 0; b < 2; ++b) u[a][b] = fma(c2k1, S1[a][b ^ 1], c2k0 * S1[a][b]);
+      for (int a = 0; a < 2; ++a)
 #pragma unroll
-        for (int a = 0; a < 2; ++a)
-#pragma unroll
-          for (int b = 0; b < 2; ++b) {
-            T& y = Y[b0][b1][a][b];
-            y = a0 == 0 ? fma(cA[a], u[a][b], cA[2 + a] * u[a ^ 1][b])
-                        : fma(cA[a], u[a][b], fma(cA[2 + a], u[a ^ 1][b], y));
-          }
-      }
+        for (int b = 0; b < 2; ++b) {
+          T& y = k == 0 ? YO[a][b] : Yh[k == 0 ? 0 : k - 1][a][b];
+          y = a0 == 0 ? fma(cA[a], u[a][b], cA[2 + a] * u[a ^ 1][b])
+                      : fma(cA[a], u[a][b], fma(cA[2 + a], u[a ^ 1][b], y));
+        }
+    }
   }
   T S2[2][2][2];                                           // [ff][q0][q2]
   {
@@ -539,9 +553,10 @@ __device__ __forceinline__ void quad_pass(T* stage, T pI, T pE, const RegMsgs<T,
       for (int a = 0; a < 2; ++a)
 #pragma unroll
         for (int b = 0; b < 2; ++b)
-          S2[f][a][b] = fma(bm[1][1][f], Y[1][1][a][b],
-                            fma(bm[1][0][f], Y[1][0][a][b],
-                                fma(bm[0][1][f], Y[0][1][a][b], bm[0][0][f] * Y[0][0][a][b])));
+          S2[f][a][b] = fma(bm[1][1][f], h ? Yh[1][a][b] : YO[a][b],
+                            fma(bm[1][0][f], h ? Yh[0][a][b] : YO[a][b],
+                                fma(bm[0][1][f], h ? YO[a][b] : Yh[1][a][b],
+                                    bm[0][0][f] * (h ? YO[a][b] : Yh[0][a][b]))));
   }
   // Column 3 (qubits at 1, 3): the upper leg e is tied to r0, the lower leg f
   // closes against B's expected value.
@@ -574,187 +589,6 @@ __device__ __forceinline__ void quad_pass(T* stage, T pI, T pE, const RegMsgs<T,
       for (int b = 0; b < 2; ++b) sj[at(a, b)] = out[a][b];
     __syncwarp();
   }
-}
-
-// The update of eight 4 x 4 blocks in FP64, with as few FP64 operations as the
-// structure allows (the FP64 pipe is the bound; selects cost nothing beside
-// it).  A qubit's table is pi(X) everywhere but at its id, so with tables
-// divided by pi(X) (a factor of the message, which the normalisation takes
-// out) a butterfly is the pair's sum, plus (rho - 1) times one of the pair
-// where the id's beta matches: rows share sums, half of the rows need no
-// multiply-add, and of column 1's four (b0, b1) products three are the value
-// itself.  170 operations a lane (four rows) and contraction against 264 for
-// quad_pass's; with inv_norm, 230 against 372 for an update.  1000 syndromes
-// at d = 11, p = 0.10: 16.4 -> 12.6 ms, FP64 pipe 87 % busy.
-template <bool GM>
-__device__ __forceinline__ void quad_update64(double* stage, const RegMsgs<double, GM>& ms,
-                                              const RegJob<double, GM>& jb, int lane, const RegUpd<double>& upd) {
-  using T = double;
-  const int r1 = (lane >> 1) & 1, r3 = lane & 1, g = lane >> 2;
-  const unsigned tq = jb.id ^ (r1 ? 0x0505u : 0u) ^ (r3 ? 0x0484u : 0u);   // as in quad_pass
-  auto beta = [&](int f) { return (bool)((tq >> (2 * f)) & 1u); };
-  auto alpha = [&](int f) { return (bool)((tq >> (2 * f + 1)) & 1u); };
-  const T rho = upd.rho, rm1 = upd.rho_m1;
-  T* sj = stage + (g << 4);
-  {
-    const T* A = ms.at(jb.cq, jb.up());
-    T a[8];                                                // [a1][v][e] of a0 = r3
-    if (jb.srev()) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) a[i] = A[r3 + 2 * (i >> 2) + 4 * ((i >> 1) & 1) + 8 * (i & 1)];
-    } else {
-      T lo[4], hi[4];
-      vcopy4(A + 8 * r3, lo);
-      vcopy4(A + 8 * r3 + 4, hi);
-#pragma unroll
-      for (int i = 0; i < 4; ++i) { a[i] = lo[i]; a[4 + i] = hi[i]; }
-    }
-    // [alpha][q0]: v = 0 and v = 1 of a1 = q0 ^ alpha, e = q0.
-    const T v0[4] = {a[0], a[5], a[4], a[1]}, v1[4] = {a[2], a[7], a[6], a[3]};
-    T c[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) c[i] = v0[i] + v1[i];
-    const bool al = alpha(4), be = beta(4);
-#pragma unroll
-    for (int q = 0; q < 2; ++q) {
-      const T e = fma(rm1, al ? (be ? v1[2 + q] : v0[2 + q]) : (be ? v1[q] : v0[q]), al ? c[2 + q] : c[q]);
-      c[q] = al ? c[q] : e;
-      c[2 + q] = al ? e : c[2 + q];
-    }
-    vstore4(sj + 8 * r1 + 4 * r3, c);
-  }
-  __syncwarp();
-  const RowAt at(jb.chk0(), r1, r3);
-  T S0[2][2][2];                                           // [a0][q0][q2]
-  {
-    const T* X = ms.at(jb.cq, jb.in());
-    T x[2][2], u[2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int b = 0; b < 2; ++b) x[a][b] = X[at(a, b)];
-    const bool al = alpha(1);
-    const T k = beta(1) ? 0.0 : rm1;
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      const T s = x[a][0] + x[a][1];
-#pragma unroll
-      for (int b = 0; b < 2; ++b) u[a][b] = fma(k, al ? x[a][b ^ 1] : x[a][b], s);
-    }
-    const bool al0 = alpha(0), be0 = beta(0);
-#pragma unroll
-    for (int b = 0; b < 2; ++b) {
-      const T s = u[0][b] + u[1][b];
-#pragma unroll
-      for (int a = 0; a < 2; ++a) {
-        const T e = fma(rm1, al0 ? u[a ^ 1][b] : u[a][b], s);
-        S0[0][a][b] = be0 ? s : e;
-        S0[1][a][b] = be0 ? e : s;
-      }
-    }
-  }
-  // The rows with r0 ^ r2 = beta: (r, r ^ beta), r = 0, 1.
-  auto butterfly = [&](int f, const T (&o)[2][2], T (&t)[2][2]) {   // over r1, beta = r0 ^ r2
-    const bool al = alpha(f), be = beta(f);
-    T p[2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        p[a][b] = shx(o[a][b], 2);
-        t[a][b] = o[a][b] + p[a][b];
-      }
-#pragma unroll
-    for (int r = 0; r < 2; ++r) {
-      const T w = be ? (al ? p[r][r ^ 1] : o[r][r ^ 1]) : (al ? p[r][r] : o[r][r]);
-      const T e = fma(rm1, w, be ? t[r][r ^ 1] : t[r][r]);
-      t[r][r] = be ? t[r][r] : e;
-      t[r][r ^ 1] = be ? e : t[r][r ^ 1];
-    }
-  };
-  // Column 1's lower qubit scales T_h, h = its id's b0, where b1 ^ r2 is its
-  // beta: b1 = beta scales row r2 = 0 (P), b1 = 1 - beta row r2 = 1 (Q); the
-  // other b0 (O) is the same for both b1.
-  const bool h = alpha(3), hv = beta(3);
-  const bool al5 = alpha(5);
-  const T k5 = beta(5) ? 0.0 : rm1;
-  T YO[2][2], YP[2][2], YQ[2][2];
-#pragma unroll
-  for (int a0 = 0; a0 < 2; ++a0) {
-    T cA[4];
-    vcopy4(sj + 8 * r1 + 4 * a0, cA);
-    T t[2][2];
-    butterfly(2, S0[a0], t);
-    T uO[2][2], uP[2][2], uQ[2][2];
-#pragma unroll
-    for (int a = 0; a < 2; ++a) {
-      T th[2], to[2], rh[2];
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        th[b] = __shfl_sync(kFull, t[a][b], (lane & ~1) | (h ? 1 : 0));
-        to[b] = __shfl_sync(kFull, t[a][b], (lane & ~1) | (h ? 0 : 1));
-        rh[b] = rho * th[b];
-      }
-      const T sO = to[0] + to[1], sP = rh[0] + th[1], sQ = th[0] + rh[1];
-      uO[a][0] = fma(k5, al5 ? to[1] : to[0], sO);
-      uO[a][1] = fma(k5, al5 ? to[0] : to[1], sO);
-      uP[a][0] = fma(k5, al5 ? th[1] : rh[0], sP);
-      uP[a][1] = fma(k5, al5 ? rh[0] : th[1], sP);
-      uQ[a][0] = fma(k5, al5 ? rh[1] : th[0], sQ);
-      uQ[a][1] = fma(k5, al5 ? th[0] : rh[1], sQ);
-    }
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        if (a0 == 0) {
-          YO[a][b] = fma(cA[a], uO[a][b], cA[2 + a] * uO[a ^ 1][b]);
-          YP[a][b] = fma(cA[a], uP[a][b], cA[2 + a] * uP[a ^ 1][b]);
-          YQ[a][b] = fma(cA[a], uQ[a][b], cA[2 + a] * uQ[a ^ 1][b]);
-        } else {
-          YO[a][b] = fma(cA[a], uO[a][b], fma(cA[2 + a], uO[a ^ 1][b], YO[a][b]));
-          YP[a][b] = fma(cA[a], uP[a][b], fma(cA[2 + a], uP[a ^ 1][b], YP[a][b]));
-          YQ[a][b] = fma(cA[a], uQ[a][b], fma(cA[2 + a], uQ[a ^ 1][b], YQ[a][b]));
-        }
-      }
-  }
-  T uu[2][2];
-  {
-    const T* B = ms.at(jb.cq, jb.lo());
-    T bm[2][2][2];                                         // B[b0 b1 r3 ff]
-    if (jb.srev()) {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) bm[i >> 2][(i >> 1) & 1][i & 1] = B[(i >> 2) + 2 * ((i >> 1) & 1) + 4 * r3 + 8 * (i & 1)];
-    } else {
-#pragma unroll
-      for (int i = 0; i < 8; ++i) bm[i >> 2][(i >> 1) & 1][i & 1] = B[4 * (i >> 1) + 2 * r3 + (i & 1)];
-    }
-    T S2[2][2][2];                                         // [ff][q0][q2]
-#pragma unroll
-    for (int f = 0; f < 2; ++f) {
-      const T bO = (h ? bm[0][0][f] : bm[1][0][f]) + (h ? bm[0][1][f] : bm[1][1][f]);
-      const T b0 = h ? bm[1][0][f] : bm[0][0][f], b1 = h ? bm[1][1][f] : bm[0][1][f];
-      const T bP = hv ? b1 : b0, bQ = hv ? b0 : b1;
-#pragma unroll
-      for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) S2[f][a][b] = fma(bQ, YQ[a][b], fma(bP, YP[a][b], bO * YO[a][b]));
-    }
-    const bool al = alpha(7), be = beta(7);
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-      for (int b = 0; b < 2; ++b) {
-        const T z0 = S2[0][a][b], z1 = S2[1][a][b];
-        const T p0 = shx(z0, 1), p1 = shx(z1, 1);
-        const bool one = be != (b == 1);                   // the id's beta against r2: z1 or z0
-        uu[a][b] = fma(rm1, one ? (al ? p1 : z1) : (al ? p0 : z0), (z0 + p0) + (z1 + p1));
-      }
-  }
-  T out[2][2];
-  butterfly(6, uu, out);
-  reg_update16(out, ms, jb, at, (lane & 3) == 0, upd);
-  __syncwarp();
 }
 
 // Eight blocks of one column of 4 nodes: as quad_pass's column 0, both side
@@ -918,14 +752,242 @@ __device__ __forceinline__ void dot_pass(T* stage, T pI, T pE, const RegMsgs<T, 
   __syncwarp();
 }
 
+// ---------------------------------------------------------------------------
+// Updates of the blocks three nodes wide or high that the last block row and
+// column hold at even d, in the roundings of the node-by-node form
+// (fused_sweep, as compiled), whose bits they reproduce: of a butterfly's two
+// terms the input with row bit 1 is the fused one.  Through that form these
+// blocks, a quarter of the messages at d = 12, took most of the time.  Eight
+// jobs a pass, four lanes each, as above.  2000 syndromes at d = 12, p = 0.10:
+// 11.1 -> 2.9 ms.
+
+// Table entry g[al][be] of the qubit in field f.
+template <typename T>
+__device__ __forceinline__ T qat(unsigned id, int f, int al, int be, T pI, T pE) {
+  return ((id >> (2 * f)) & 3u) == (unsigned)((al << 1) | be) ? pI : pE;
+}
+// Butterfly over a row bit held by lane bit `mask`, r the lane's own.
+template <typename T>
+__device__ __forceinline__ T lane_bf(T x, int mask, int r, T g0, T g1) {
+  const T y = shx(x, mask);
+  return fma(r ? x : y, r ? g0 : g1, r ? y * g1 : x * g0);
+}
+// First qubit of a column, its row bit in registers: inputs x[l], output r,
+// the upper leg u given (in the table entries) or summed.
+template <typename T>
+__device__ __forceinline__ T reg_bf(T x0, T x1, int r, T g0, T g1) {
+  return r ? fma(x1, g0, x0 * g1) : fma(x1, g1, x0 * g0);
+}
+template <typename T>
+__device__ __forceinline__ T reg_bf4(T x00, T x01, T x10, T x11, T ga, T gb, T gc, T gd) {   // x[l][u]
+  return fma(x11, gd, fma(x10, gc, fma(x00, ga, x01 * gb)));
+}
+
+// The update of an 8-entry vector out[q0], (r1, r2) = lane bits: reg_update16
+// with sums over r0, r1, r2.
+template <typename T, bool GM>
+__device__ __forceinline__ void reg_update8(const T (&out)[2], const RegMsgs<T, GM>& ms, const RegJob<T, GM>& jb,
+                                            int lane, const RegUpd<T>& up) {
+  T* old = ms.out(jb.cq, jb.out()) + (lane & 3);
+  auto sum = [&](T a, T b) {
+    T v = radd(a, b);
+    v = radd(v, shx(v, 2));
+    return radd(v, shx(v, 1));
+  };
+  const T y0 = old[0], y1 = old[4];
+  const T i1 = inv_norm(sum(out[0] * out[0], out[1] * out[1]));
+  T x0 = fma(up.one_m_eta, out[0] * i1, up.eta * y0), x1 = fma(up.one_m_eta, out[1] * i1, up.eta * y1);
+  const T i2 = inv_norm(sum(x0 * x0, x1 * x1));
+  x0 = x0 * i2;
+  x1 = x1 * i2;
+  T term;
+  if constexpr (sizeof(T) == 4) {
+    const T t0 = x0 - y0, t1 = x1 - y1;
+    const T sq = sum(t0 * t0, t1 * t1);
+    term = sq * fma(T(-0.5), sq, T(2));
+  } else {
+    const T o = sum(x0 * y0, x1 * y1);
+    term = fma(T(-2) * o, o, T(2));
+  }
+  if (jb.on) {
+    old[0] = x0;
+    old[4] = x1;
+    if ((lane & 3) == 0) up.ovl[jb.cq * up.M + jb.out()] = term;
+  }
+}
+
+// 4 x 3: columns Q (qubits at 0, 2), C (1, 3), Q; column 0 lies on the grid
+// border (no incoming message), the lower side has a message, the upper one
+// unless the block is in the first row.  (r1, r3) = lane bits, r0, r2 = q0, q2.
+template <typename T, bool GM>
+__device__ __forceinline__ void pass43(T pI, T pE, const RegMsgs<T, GM>& ms, const RegJob<T, GM>& jb, int lane,
+                                       const RegUpd<T>& upd) {
+  const int r1 = (lane >> 1) & 1, r3 = lane & 1;
+  const unsigned id = jb.id;
+  const bool a = jb.up() < ms.M, srev = jb.srev();
+  const T* A = ms.at(jb.cq, jb.up());
+  const int s0 = srev ? 1 : 4, s2 = srev ? 4 : 1;            // strides of side legs 0 and 2 (leg 1: 2)
+  const T* B = ms.at(jb.cq, jb.lo()) + (r3 ? s2 : 0);        // only its leg 2 = r3 reaches column 2's rows
+  // Column 0: the incoming side is e_0 at the qubits, so each output is a
+  // product of two table entries.  Column 1's upper side message over a0
+  // (v = r0) leaves its leg 2.
+  T x[2][2][2];                                              // [a2][q0][q2]
+#pragma unroll
+  for (int q0 = 0; q0 < 2; ++q0)
+#pragma unroll
+    for (int q2 = 0; q2 < 2; ++q2) {
+      const T g2 = qat(id, 1, q2, r1 ^ r3, pI, pE);
+      const T e0 = qat(id, 0, q0, r1, pI, pE) * g2, e1 = qat(id, 0, q0, r1 ^ 1, pI, pE) * g2;   // a0 = 0, 1
+#pragma unroll
+      for (int a2 = 0; a2 < 2; ++a2) {
+        const T* m = A + 2 * q0 + (a2 ? s2 : 0);
+        x[a2][q0][q2] = a ? fma(m[s0], e1, m[0] * e0) : (a2 ? T(0) : e0);
+      }
+    }
+  // Qubit 1, then qubit 3 with l3 = b0, and the lower message over b0 and w.
+  T z[2][2][2];
+  const T b00 = B[0], b01 = B[2], b10 = B[s0], b11 = B[s0 + 2];
+#pragma unroll
+  for (int q0 = 0; q0 < 2; ++q0)
+#pragma unroll
+    for (int q2 = 0; q2 < 2; ++q2) {
+      const T g0 = qat(id, 2, 0, q0 ^ q2, pI, pE), g1 = qat(id, 2, 1, q0 ^ q2, pI, pE);
+      const T h00 = qat(id, 3, r3, q2, pI, pE), h01 = qat(id, 3, r3, q2 ^ 1, pI, pE);           // b0 = 0; w = 0, 1
+      const T h10 = qat(id, 3, r3 ^ 1, q2, pI, pE), h11 = qat(id, 3, r3 ^ 1, q2 ^ 1, pI, pE);   // b0 = 1
+#pragma unroll
+      for (int a2 = 0; a2 < 2; ++a2) {
+        const T t = lane_bf(x[a2][q0][q2], 2, r1, g0, g1);
+        const T t0 = __shfl_sync(kFull, t, lane & ~1), t1 = __shfl_sync(kFull, t, lane | 1);
+        const T v = fma(b00, t0 * h00, b01 * (t0 * h01));
+        z[a2][q0][q2] = radd(v, fma(b10, t1 * h10, b11 * (t1 * h11)));
+      }
+    }
+  // Column 2: qubit 0 with its upper leg a2 summed, then qubit 2.
+  const T g0 = qat(id, 4, 0, r1, pI, pE), g1 = qat(id, 4, 1, r1, pI, pE);
+  const T h0 = qat(id, 4, 0, r1 ^ 1, pI, pE), h1 = qat(id, 4, 1, r1 ^ 1, pI, pE);
+  const T k0 = qat(id, 5, 0, r1 ^ r3, pI, pE), k1 = qat(id, 5, 1, r1 ^ r3, pI, pE);
+  T out[2][2];
+#pragma unroll
+  for (int q0 = 0; q0 < 2; ++q0) {
+    T y[2];
+#pragma unroll
+    for (int q2 = 0; q2 < 2; ++q2)
+      y[q2] = q0 ? reg_bf4(z[0][0][q2], z[1][0][q2], z[0][1][q2], z[1][1][q2], g1, h1, g0, h0)
+                 : reg_bf4(z[0][0][q2], z[1][0][q2], z[0][1][q2], z[1][1][q2], g0, h0, g1, h1);
+    out[q0][0] = fma(y[1], k1, y[0] * k0);
+    out[q0][1] = fma(y[1], k0, y[0] * k1);
+  }
+  reg_update16(out, ms, jb, RowAt(false, r1, r3), (lane & 3) == 0, upd);
+  __syncwarp();
+}
+
+// 3 x 4 (chains of three nodes ending on the grid border: no lower message,
+// the upper one always), and 3 x 3 (the corner block: no incoming message
+// either).  r0 = q0, (r1, r2) = lane bits.  A qubit at position 2 has no lower
+// leg (beta = r1), a check there no constraint.
+template <typename T, bool GM, bool CORNER>
+__device__ __forceinline__ void pass3(T pI, T pE, const RegMsgs<T, GM>& ms, const RegJob<T, GM>& jb, int lane,
+                                      const RegUpd<T>& upd) {
+  const int r1 = (lane >> 1) & 1, r2 = lane & 1;
+  const unsigned id = jb.id;
+  const bool srev = jb.srev(), chk0 = jb.chk0();
+  const T* A = ms.at(jb.cq, jb.up());
+  auto bf1 = [&](T x, int f, int q0) {                       // qubit 1 of a C column, field f
+    return lane_bf(x, 2, r1, qat(id, f, 0, q0 ^ r2, pI, pE), qat(id, f, 1, q0 ^ r2, pI, pE));
+  };
+  auto bf2 = [&](T x, int f) {                               // qubit 2 of a Q column, field f
+    return lane_bf(x, 1, r2, qat(id, f, 0, r1, pI, pE), qat(id, f, 1, r1, pI, pE));
+  };
+  auto first4 = [&](T x00, T x01, T x10, T x11, int f, int r) {   // qubit 0 with u summed, x[l][u]
+    const T ga = qat(id, f, r, r1, pI, pE), gb = qat(id, f, r, r1 ^ 1, pI, pE);
+    const T gc = qat(id, f, r ^ 1, r1, pI, pE), gd = qat(id, f, r ^ 1, r1 ^ 1, pI, pE);
+    return reg_bf4(x00, x01, x10, x11, ga, gb, gc, gd);
+  };
+  T out[2] = {T(0), T(0)};
+  if constexpr (CORNER) {
+    const int s0 = srev ? 1 : 4, s2 = srev ? 4 : 1;          // strides of side legs 0 and 2 (leg 1: 2)
+    T z[2][2];                                               // [a2][r0]
+#pragma unroll
+    for (int q0 = 0; q0 < 2; ++q0) {
+      const T g2 = qat(id, 1, r2, r1, pI, pE);
+      const T e0 = qat(id, 0, q0, r1, pI, pE) * g2, e1 = qat(id, 0, q0, r1 ^ 1, pI, pE) * g2;   // a0 = 0, 1
+#pragma unroll
+      for (int a2 = 0; a2 < 2; ++a2) {
+        const T* m = A + 2 * q0 + (a2 ? s2 : 0);
+        z[a2][q0] = bf1(fma(m[s0], e1, m[0] * e0), 2, q0);
+      }
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) out[r] = bf2(first4(z[0][0], z[1][0], z[0][1], z[1][1], 4, r), 5);
+  } else {
+    const int s0 = srev ? 1 : 8, s1 = srev ? 2 : 4, s2 = srev ? 4 : 2, s3 = srev ? 8 : 1;   // strides of the side legs
+    const T* X = ms.at(jb.cq, jb.in()) + (lane & 3);
+    const T x0 = X[0], x1 = X[4];
+    // The lists keep the two forms apart, so a pass mostly runs one; where it
+    // holds both, each job keeps its own.
+    if (__any_sync(kFull, !chk0)) {  // Q, C, Q, C
+      T y[2][2];                                             // [a0][r0], a0 = u
+#pragma unroll
+      for (int a0 = 0; a0 < 2; ++a0) {
+        const T g0 = qat(id, 0, 0, a0 ^ r1, pI, pE), g1 = qat(id, 0, 1, a0 ^ r1, pI, pE);
+#pragma unroll
+        for (int r = 0; r < 2; ++r) y[a0][r] = bf1(bf2(reg_bf(x0, x1, r, g0, g1), 1), 2, r);
+      }
+      // The message over a0 (a1 = l0) and, at qubit 0, its leg 2 = u; leg 3 = r0 of the last column.
+      T w[2][2][2];                                          // [leg 3][u][l0]
+#pragma unroll
+      for (int l0 = 0; l0 < 2; ++l0)
+#pragma unroll
+        for (int u = 0; u < 2; ++u)
+#pragma unroll
+          for (int a3 = 0; a3 < 2; ++a3) {
+            const T* m = A + (l0 ? s1 : 0) + (u ? s2 : 0) + (a3 ? s3 : 0);
+            w[a3][u][l0] = fma(m[s0], y[1][l0], m[0] * y[0][l0]);
+          }
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const T v = bf1(bf2(first4(w[r][0][0], w[r][1][0], w[r][0][1], w[r][1][1], 4, r), 5), 6, r);
+        out[r] = chk0 ? out[r] : v;
+      }
+    }
+    if (__any_sync(kFull, chk0)) {   // C, Q, C, Q
+      const T c0 = bf1(x0, 0, 0), c1 = bf1(x1, 0, 1);        // a0 = r0
+      T w[2][2];                                             // [leg 3][r0]
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        T y[2][2];                                           // [a0][a1]: qubit 0 with l0 = a0, a1 = u
+#pragma unroll
+        for (int a0 = 0; a0 < 2; ++a0)
+#pragma unroll
+          for (int a1 = 0; a1 < 2; ++a1)
+            y[a0][a1] = bf2((a0 ? c1 : c0) * qat(id, 2, a0 ^ r, a1 ^ r1, pI, pE), 3);
+#pragma unroll
+        for (int a3 = 0; a3 < 2; ++a3) {
+          const T* m = A + (r ? s2 : 0) + (a3 ? s3 : 0);     // leg 2 = r0
+          const T v = fma(m[s0 + s1], y[1][1], fma(m[s0], y[1][0], fma(m[s1], y[0][1], m[0] * y[0][0])));
+          w[a3][r] = bf1(v, 4, r);
+        }
+      }
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const T v = bf2(first4(w[0][0], w[1][0], w[0][1], w[1][1], 6, r), 7);
+        out[r] = chk0 ? v : out[r];
+      }
+    }
+  }
+  reg_update8(out, ms, jb, lane, upd);
+  __syncwarp();
+}
+
 template <typename T, bool GM, bool UPD, int SHAPE>
 __device__ __forceinline__ void reg_pass(T* stage, T pI, T pE, const RegMsgs<T, GM>& ms, const RegJob<T, GM>& jb,
                                          int lane, const RegUpd<T>& upd) {
-  if constexpr (SHAPE == kShapeQuad && UPD && sizeof(T) == 8) quad_update64<GM>(stage, ms, jb, lane, upd);
-  else if constexpr (SHAPE == kShapeQuad) quad_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
+  if constexpr (SHAPE == kShapeQuad) quad_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
   else if constexpr (SHAPE == kShapeCol) col_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
   else if constexpr (SHAPE == kShapeRow) row_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
-  else dot_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
+  else if constexpr (SHAPE == kShapeDot) dot_pass<T, GM, UPD>(stage, pI, pE, ms, jb, lane, upd);
+  else if constexpr (SHAPE == kShape43) pass43<T, GM>(pI, pE, ms, jb, lane, upd);
+  else pass3<T, GM, SHAPE == kShape33>(pI, pE, ms, jb, lane, upd);
 }
 
 // Message item of job j when every message has n jobs (n = 1 .. 4).

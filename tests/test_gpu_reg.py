@@ -2,7 +2,7 @@
 (message, coset) of one shape per warp pass, so small codes leave passes
 partly empty (d = 3: one 4 x 4 block and the three one-node-wide ones), and
 cosets that stop at different iterations leave one, two or three jobs per
-message.  Against the dense oracle, with the repository's bars: |delta log P|
+message; even distances have blocks three nodes wide.  Against the dense oracle, with the repository's bars: |delta log P|
 <= 1e-9 in FP64 and 1e-3 in FP32."""
 
 import numpy as np
@@ -19,7 +19,8 @@ torch = pytest.importorskip("torch")
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("precision,tol", [("fp64", 1e-9), ("fp32", 1e-3)])
-@pytest.mark.parametrize("d,B,delta0", [(3, 3, 0.0), (3, 3, 1e-3), (5, 3, 1e-3), (7, 2, 1e-4)])
+@pytest.mark.parametrize("d,B,delta0", [(3, 3, 0.0), (3, 3, 1e-3), (4, 3, 0.0), (5, 3, 1e-3),
+                                        (6, 2, 1e-3), (7, 2, 1e-4), (8, 1, 1e-4)])
 def test_partly_filled_passes(precision, tol, d, B, delta0):
     p, iters = 0.1, 12
     _, _, S = synth.sample_syndromes(8800 + d, 0, B, d, p)
@@ -30,6 +31,8 @@ def test_partly_filled_passes(precision, tol, d, B, delta0):
             want[b, c], _, its[b, c], _ = run_naive(coset_network(Lattice(d), S[b], c, p), 4, iters, 0.1, delta0)
     first = None
     for warps, cosets, messages in ((0, 0, 0), (8, 1, 1), (8, 2, 3), (4, 2, 1), (4, 4, 1)):
+        if messages == 3 and d % 2 == 0:
+            continue                                      # odd distances only
         if messages == 3 and precision == "fp64":
             warps, cosets = 4, 2
         prm = pkg.DecoderParams(d=d, k=4, p=p, max_iter=iters, delta0=delta0, precision=precision, algorithm="fused",
@@ -48,7 +51,8 @@ def test_partly_filled_passes(precision, tol, d, B, delta0):
 @pytest.mark.gpu
 @pytest.mark.parametrize("d,B", [(3, 700), (5, 1), (5, 80), (7, 200), (9, 400), (11, 39), (11, 77), (11, 153), (11, 305),
                                  (11, 2500), (13, 400), (17, 320), (21, 160), (27, 160), (29, 3), (29, 160), (41, 2),
-                                 (53, 2)])
+                                 (53, 2), (2, 700), (4, 1), (6, 80), (8, 160), (12, 320), (12, 1000), (20, 400), (26, 3),
+                                 (30, 160), (40, 2), (52, 2)])
 def test_default_kernel_of_every_size_gives_the_same_bits(d, B):
     # The default launch takes a kernel by geometry and batch; each gives the
     # bits of a kernel asked for by shape (messages in shared memory, or in
