@@ -13,7 +13,7 @@ int smem_bytes_for(const Geo& g, int M, int warps = kWarps) {
 }
 
 template <typename T, int NW>
-cudaError_t launch_decode_nw(const LaunchArgs& a, cudaStream_t st) {
+cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) {
   KArgs<T> k;
   k.geo = a.geo; k.M = a.M; k.D = a.D; k.max_iter = a.max_iter; k.arena_elems = a.arena_elems;
   k.p = a.p; k.eta = a.eta; k.delta0 = a.delta0; k.delta1 = a.delta1; k.cutoff = a.cutoff;
@@ -26,34 +26,61 @@ cudaError_t launch_decode_nw(const LaunchArgs& a, cudaStream_t st) {
   auto kern = decode_kernel<T, kMaxK, kMaxD, NW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
-  const unsigned grid = (unsigned)(a.B * 4);
-  kern<<<grid, NW * 32, smem, st>>>(k);
-  return cudaGetLastError();
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = (unsigned)cluster;
+  at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(a.B * 4 * cluster));
+  cfg.blockDim = dim3(NW * 32);
+  cfg.dynamicSmemBytes = (size_t)smem;
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = cluster > 1 ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, k);
 }
 
-// Warps per CTA (one message update each): eight where they fit beside the
-// tables (the linear algebra is a chain of short dependent steps; one SM holds
-// 8 warps in FP64 either way, 16 instead of 12 in FP32), four for small
-// networks in FP64 unless SMs would stay idle (half-rounds of few messages),
-// sixteen in FP32 for batches that leave SMs idle.  FP64 d = 11: 24 syndromes
-// 285 -> 224 ms, 60: 440 -> 385; d = 5 with k = 3: 60 syndromes 19.1 ms with
-// four, 20.6 with eight, 10 syndromes 12.4 and 10.2.  FP32 d = 11: 24 syndromes
-// 95 ms with four, 59 with eight, 50 with sixteen; 300: 421, 368, 379.
+// Warps per CTA (one message update each) and CTAs per network.  The linear
+// algebra is a chain of short dependent steps, and one SM holds 8 warps in FP64
+// and 16 in FP32 (the warps' shared memory), so what a batch leaves idle goes
+// to clusters that share a network's half-round (60 updates at d = 11, 12 at
+// d = 5 with k = 3), up to a warp per update:
+// - FP64: four-warp CTAs, as many per network as are resident together, from
+//   three on; eight-warp CTAs where even those leave half the chip idle; else
+//   pairs of eight-warp CTAs (shorter rounds, a fuller last wave).
+// - FP32: eight-warp CTAs, as many per network as are resident, at least two.
+// - Half-rounds of fewer than 16 updates: four-warp CTAs, a warp per update (d =
+//   5, k = 3, 200 syndromes: 3 x 4 warps 54.5 ms, 1 x 8 56.0, 2 x 8 67.6).
+// ms, one CTA per network -> clusters: FP64 d = 11, 1 syndrome 223 -> 40 (8 x 8
+// warps; 8 x 4: 49), 5: 223 -> 59 (8 x 4; 8 x 8: 63), 12: 224 -> 84, 24: 225 ->
+// 150 (3 x 4; 2 x 8: 180), 48: 348 -> 285, 100: 558 -> 495, 200: 973 -> 927;
+// d = 5, k = 3, 1 syndrome 10.1 -> 4.9, 200: 57.9 -> 54.5.  FP32 d = 11:
+// 1 syndrome 39 -> 10, 24: 52 -> 36, 100: 147 -> 126, 300: 379 -> 343.
 template <typename T>
 cudaError_t launch_decode_t(const LaunchArgs& a, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-  const bool idle = 4 * a.B <= sms;
+  const int half = (a.M + 1) / 2;   // updates of a half-round
   auto fits = [&](int warps) { return smem_bytes_for<T>(a.geo, a.M, warps) <= kMaxSmemBytes; };
-  if constexpr (sizeof(T) == 4) {
-    if (idle && fits(16)) return launch_decode_nw<T, 16>(a, st);
-    if (fits(8)) return launch_decode_nw<T, 8>(a, st);
-  } else {
-    if ((idle || a.M >= 40) && fits(8)) return launch_decode_nw<T, 8>(a, st);
-  }
-  return launch_decode_nw<T, kWarps>(a, st);
+  auto resident = [&](int warps) {   // CTAs per network in one wave
+    const long long per_sm = kSmemPerSm / (smem_bytes_for<T>(a.geo, a.M, warps) + kSmemReservedPerCta);
+    return per_sm * sms / (4 * a.B);
+  };
+  auto cluster = [&](int warps, long long n) {
+    const long long cap = (half + warps - 1) / warps;
+    n = n < cap ? n : cap;
+    return (int)(n < 1 ? 1 : n > kMaxCluster ? kMaxCluster : n);
+  };
+  const bool small = half < 16;
+  bool four = !fits(8) || small;
+  if (sizeof(T) == 8 && !four) four = resident(4) >= 3 && !(64 * a.B <= sms && half > 4 * kMaxCluster);
+  const int warps = four ? 4 : 8;
+  const long long n = resident(warps);
+  int cs = cluster(warps, small ? kMaxCluster : n < 2 ? 2 : n);
+  if (4 * a.B * cs > 0x7fffffff) cs = 1;   // grid limit
+  return four ? launch_decode_nw<T, 4>(a, cs, st) : launch_decode_nw<T, 8>(a, cs, st);
 }
 
 template <typename T, int K>

@@ -1,12 +1,13 @@
 // Device code of the blockBP decoder (arXiv:2402.04834, Sec. III.D,
 // Algorithm 1, Remarks 2-8, Lemma 1) for sm_103a.
 //
-// One CTA decodes one (syndrome, coset) pair from start to end: it builds
-// the coset frame f_s * L (Algorithm 1, first steps), keeps the MPS messages
-// of all M directed block edges in a global-memory arena, runs the
-// chessboard schedule (Remark 8) with one warp per message update and a
-// __syncthreads() between half-rounds, evaluates Delta (Remark 4) and the
-// Bethe read-out of Lemma 1.  No CTA ever waits on another CTA.
+// One CTA, or a cluster of them in a small batch, decodes one (syndrome,
+// coset) pair from start to end: it builds the coset frame f_s * L (Algorithm
+// 1, first steps), keeps the MPS messages of all M directed block edges in a
+// global-memory arena, runs the chessboard schedule (Remark 8) with one warp
+// per message update and a barrier of the cluster between half-rounds,
+// evaluates Delta (Remark 4) and the Bethe read-out of Lemma 1.  No CTA ever
+// waits on one outside its cluster.
 //
 // A warp owns a shared-memory workspace holding the running boundary MPS of
 // one block contraction.  The linear algebra is warp-cooperative on that
@@ -48,6 +49,29 @@ __device__ __forceinline__ bool dev_check(bool ok, int* flags) {
     }
   }
   return true;
+}
+
+// The cluster of CTAs that shares one network (one CTA when launched without
+// one): its size, this CTA's rank, a peer's copy of a shared-memory object, and
+// a barrier that also orders global memory between its CTAs.
+__device__ __forceinline__ int cluster_size() {
+  unsigned n;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
+  return (int)n;
+}
+__device__ __forceinline__ int cluster_rank() {
+  unsigned r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return (int)r;
+}
+template <typename P>
+__device__ __forceinline__ P* cluster_peer(P* p, int rank) {
+  unsigned long long q;
+  asm("mapa.u64 %0, %1, %2;" : "=l"(q) : "l"((unsigned long long)p), "r"(rank));
+  return reinterpret_cast<P*>(q);
+}
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 template <typename T> struct Eps;
@@ -165,7 +189,8 @@ struct Ctx {
   int8_t* dims;            // [M][K+1] bond dims of every message
   T* arena;                // this CTA's message arena
   const T* e0;             // the trivial border site (1, 0)
-  int* cta_flags;
+  int* cta_flags;       // rank 0's, when a cluster of CTAs shares the network
+  int cluster;          // CTAs that share the network
 };
 
 // ---------------------------------------------------------------------------
@@ -1164,13 +1189,19 @@ __device__ __noinline__ void store_msg(WarpWS<T, K, DM>& ws, const Ctx<T, K>& c,
   T* base = c.arena + c.msg_off[idx];
   for (int s = 0; s < w; ++s)
     warp_copy(base + msg_site_offset(s, w, c.D), ws.psi[s], ws.bond[s] * 2 * ws.bond[s + 1], lane);
-  int8_t* dm = c.dims + idx * (K + 1);
-  for (int s = lane; s <= w; s += 32) dm[s] = (int8_t)ws.bond[s];
+  for (int r = 0; r < c.cluster; ++r) {
+    int8_t* dm = cluster_peer(c.dims, r) + idx * (K + 1);
+    for (int s = lane; s <= w; s += 32) dm[s] = (int8_t)ws.bond[s];
+  }
   __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
-// The decoder kernel: one CTA per (syndrome, coset).
+// The decoder kernel: one cluster of CTAs per (syndrome, coset), a single CTA
+// where the batch fills the chip.  Messages are in the global arena; the tables
+// are built in every CTA, message bond dimensions and overlaps are written to
+// every CTA's copy, and the item counter, the flags and the read-out terms are
+// those of rank 0, so results do not depend on the cluster size.
 template <typename T, int K, int DM, int NW>
 __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1194,10 +1225,13 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
   WS* wsa = reinterpret_cast<WS*>(smem + Lo.ws);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const long long cta = blockIdx.x;
+  const int CS = cluster_size(), cr = cluster_rank();
+  const long long cta = blockIdx.x / CS;
   const long long shot = cta >> 2;
   const int coset = (int)(cta & 3);
   T* arena = a.arena + cta * (long long)a.arena_elems;
+  int* misc0 = cluster_peer(misc, 0);
+  double* rlog0 = cluster_peer(rlog, 0);
 
   // Syndrome and the coset frame f_s * L (Algorithm 1; pure-error strings to
   // the right / bottom boundary, logicals on row 0 / column 0).
@@ -1246,7 +1280,8 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
   c.cutoff2 = a.cutoff2_w;
   c.pI = a.pI_w; c.pE = a.pE_w;
   c.frame = frame; c.msg_of = msg_of; c.msg_off = msg_off; c.dims = dims;
-  c.arena = arena; c.e0 = e0; c.cta_flags = &misc[1];
+  c.arena = arena; c.e0 = e0; c.cta_flags = &misc0[1];
+  c.cluster = CS;
 
   // Remark 2: uniform initial messages, bond 1, every site (1, 1)/sqrt(2).
   const T u = (T)0.70710678118654752440;
@@ -1254,13 +1289,13 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
     const int key = meta[idx];
     const int w = g.side_len(key / 4 / nb, (key / 4) % nb, key & 3);
     T* base = arena + msg_off[idx];
-    for (int s = lane; s < w; s += 32) {
+    for (int s = lane; s < w && idx % CS == cr; s += 32) {
       T* site = base + msg_site_offset(s, w, a.D);
       site[0] = u; site[1] = u;
     }
     for (int s = lane; s <= w; s += 32) dims[idx * (K + 1) + s] = 1;
   }
-  __syncthreads();
+  cluster_barrier();
 
   WS& ws = wsa[warp];
   double delta = 0.0;
@@ -1271,11 +1306,11 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
       const int16_t* lst = work + color * M;
       for (;;) {
         int item = 0;
-        if (lane == 0) item = atomicAdd(&misc[0], 1);
+        if (lane == 0) item = atomicAdd(&misc0[0], 1);
         item = __shfl_sync(kFull, item, 0);
         if (item >= nwork) break;
         const int idx = lst[item];
-        if (!dev_check(idx >= 0 && idx < M, &misc[1])) continue;
+        if (!dev_check(idx >= 0 && idx < M, &misc0[1])) continue;
         const int key = meta[idx];
         const int I = key / 4 / nb, J = (key / 4) % nb, dir = key & 3;
         const Frame f = make_frame(c, I, J, dir);
@@ -1284,11 +1319,11 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
         const double o = mps_overlap(ws, f.h, [&](int s) { return psi_site(ws, s); },
                                      [&](int s) { return msg_site(c, idx, f.h, s, false); }, lane);
         store_msg(ws, c, idx, f.h, lane);
-        if (lane == 0) ovl[idx] = o;
+        if (lane < CS) cluster_peer(ovl, lane)[idx] = o;
       }
-      __syncthreads();
-      if (tid == 0) misc[0] = 0;
-      __syncthreads();
+      cluster_barrier();
+      if (tid == 0) misc[0] = 0;   // only rank 0's counts
+      cluster_barrier();
     }
     // Remark 4: Delta = sqrt(sum_i 2 - 2 <m_i^t | m_i^(t-1)>^2) / M.
     if (warp == 0) {
@@ -1313,12 +1348,12 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
     misc[4] = nedge;
     misc[0] = 0;
   }
-  __syncthreads();
+  cluster_barrier();
   nedge = misc[4];
   const int nblk = nb * nb;
   for (;;) {
     int item = 0;
-    if (lane == 0) item = atomicAdd(&misc[0], 1);
+    if (lane == 0) item = atomicAdd(&misc0[0], 1);
     item = __shfl_sync(kFull, item, 0);
     if (item >= nblk + nedge) break;
     if (item < nblk) {
@@ -1326,32 +1361,32 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
       const Frame f = make_frame(c, I, J, kDirR);
       const double ls = block_sweep(ws, c, f, true, lane);
       const int right = J + 1 < nb ? msg_index(c, I, J + 1, kDirL) : -1;
-      if (!dev_check(right >= -1 && right < M, &misc[1])) continue;
+      if (!dev_check(right >= -1 && right < M, &misc0[1])) continue;
       const double z = mps_overlap(ws, f.h, [&](int s) { return psi_site(ws, s); },
                                    [&](int s) { return msg_site(c, right, f.h, s, false); }, lane);
       if (lane == 0) {
-        rlog[item] = ls + log(fabs(z));
-        if (!(z > 0.0)) atomicOr(&misc[1], kFlagBlock);
+        rlog0[item] = ls + log(fabs(z));
+        if (!(z > 0.0)) atomicOr(&misc0[1], kFlagBlock);
       }
     } else {
       const int e = item - nblk;
       const int idx = work[e];
-      if (!dev_check(idx >= 0 && idx < M, &misc[1])) continue;
+      if (!dev_check(idx >= 0 && idx < M, &misc0[1])) continue;
       const int key = meta[idx];
       const int I = key / 4 / nb, J = (key / 4) % nb, dir = key & 3;
       const int other = dir == kDirR ? msg_index(c, I, J + 1, kDirL) : msg_index(c, I + 1, J, kDirU);
-      if (!dev_check(other >= 0 && other < M, &misc[1])) continue;
+      if (!dev_check(other >= 0 && other < M, &misc0[1])) continue;
       const int w = g.side_len(I, J, dir);
       const double o = mps_overlap(ws, w, [&](int s) { return msg_site(c, idx, w, s, false); },
                                    [&](int s) { return msg_site(c, other, w, s, false); }, lane);
       if (lane == 0) {
-        rlog[item] = -log(fabs(o));
-        if (!(o > 0.0)) atomicOr(&misc[1], kFlagOverlap);
+        rlog0[item] = -log(fabs(o));
+        if (!(o > 0.0)) atomicOr(&misc0[1], kFlagOverlap);
       }
     }
   }
-  __syncthreads();
-  if (warp == 0) {
+  cluster_barrier();
+  if (cr == 0 && warp == 0) {
     double acc = 0.0;
     for (int i = lane; i < nblk + nedge; i += 32) acc += rlog[i];
     acc = warp_sum(acc);

@@ -11,10 +11,13 @@
 namespace bbp {
 
 // Compile-time capacity of the instances: block side k <= kMaxK and bond
-// dimension D <= kMaxD; kWarps warps (message updates in flight) per CTA.
+// dimension D <= kMaxD; kWarps warps (message updates in flight) of the
+// smallest CTA, which decides what is accepted; kMaxCluster CTAs per network
+// (the portable cluster size).
 constexpr int kMaxK = 4;
 constexpr int kMaxD = 8;
 constexpr int kWarps = 4;
+constexpr int kMaxCluster = 8;
 
 struct LaunchArgs {
   Geo geo;
