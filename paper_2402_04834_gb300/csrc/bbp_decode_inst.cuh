@@ -7,12 +7,12 @@
 
 namespace bbp {
 
-template <typename T>
+template <typename T, int DM = kMaxD>
 int smem_bytes_for(const Geo& g, int M, int warps = kWarps) {
-  return cta_layout(g, M, kMaxK, warps, (int)sizeof(WarpWS<T, kMaxK, kMaxD>)).total;
+  return cta_layout(g, M, kMaxK, warps, (int)sizeof(WarpWS<T, kMaxK, DM>)).total;
 }
 
-template <typename T, int NW>
+template <typename T, int DM, int NW>
 cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) {
   KArgs<T> k;
   k.geo = a.geo; k.M = a.M; k.D = a.D; k.max_iter = a.max_iter; k.arena_elems = a.arena_elems;
@@ -22,8 +22,8 @@ cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) 
   k.init_msgs = nullptr; k.final_msgs = nullptr;
   k.n_items = 0; k.slot_elems = 0;
   set_working(k);
-  const int smem = smem_bytes_for<T>(a.geo, a.M, NW);
-  auto kern = decode_kernel<T, kMaxK, kMaxD, NW>;
+  const int smem = smem_bytes_for<T, DM>(a.geo, a.M, NW);
+  auto kern = decode_kernel<T, kMaxK, DM, NW>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute at[1];
@@ -42,7 +42,8 @@ cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) 
 
 // Warps per CTA (one message update each) and CTAs per network.  The linear
 // algebra is a chain of short dependent steps, and one SM holds 8 warps in FP64
-// and 16 in FP32 (the warps' shared memory), so what a batch leaves idle goes
+// and 16 in FP32 (the warps' shared memory; 16 in FP64 with DM = 4 by the
+// registers), so what a batch leaves idle goes
 // to clusters that share a network's half-round (60 updates at d = 11, 12 at
 // d = 5 with k = 3), up to a warp per update:
 // - FP64: four-warp CTAs, as many per network as are resident together, from
@@ -56,17 +57,17 @@ cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) 
 // 150 (3 x 4; 2 x 8: 180), 48: 348 -> 285, 100: 558 -> 495, 200: 973 -> 927;
 // d = 5, k = 3, 1 syndrome 10.1 -> 4.9, 200: 57.9 -> 54.5.  FP32 d = 11:
 // 1 syndrome 39 -> 10, 24: 52 -> 36, 100: 147 -> 126, 300: 379 -> 343.
-template <typename T>
-cudaError_t launch_decode_t(const LaunchArgs& a, cudaStream_t st) {
+template <typename T, int DM>
+cudaError_t launch_decode_dm(const LaunchArgs& a, cudaStream_t st) {
   int dev = 0, sms = 0;
   cudaError_t e;
   if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int half = (a.M + 1) / 2;   // updates of a half-round
-  auto fits = [&](int warps) { return smem_bytes_for<T>(a.geo, a.M, warps) <= kMaxSmemBytes; };
-  auto resident = [&](int warps) {   // CTAs per network in one wave
-    const long long per_sm = kSmemPerSm / (smem_bytes_for<T>(a.geo, a.M, warps) + kSmemReservedPerCta);
-    return per_sm * sms / (4 * a.B);
+  auto fits = [&](int warps) { return smem_bytes_for<T, DM>(a.geo, a.M, warps) <= kMaxSmemBytes; };
+  auto resident = [&](int warps) {   // CTAs per network in one wave, 16 warps an SM
+    const long long per_sm = kSmemPerSm / (smem_bytes_for<T, DM>(a.geo, a.M, warps) + kSmemReservedPerCta);
+    return (per_sm * warps < 16 ? per_sm : 16 / warps) * sms / (4 * a.B);
   };
   auto cluster = [&](int warps, long long n) {
     const long long cap = (half + warps - 1) / warps;
@@ -80,7 +81,20 @@ cudaError_t launch_decode_t(const LaunchArgs& a, cudaStream_t st) {
   const long long n = resident(warps);
   int cs = cluster(warps, small ? kMaxCluster : n < 2 ? 2 : n);
   if (4 * a.B * cs > 0x7fffffff) cs = 1;   // grid limit
-  return four ? launch_decode_nw<T, 4>(a, cs, st) : launch_decode_nw<T, 8>(a, cs, st);
+  return four ? launch_decode_nw<T, DM, 4>(a, cs, st) : launch_decode_nw<T, DM, 8>(a, cs, st);
+}
+
+// D <= 4 in FP64 takes an instance of that capacity: 7 KB a warp instead of
+// 27, 8 columns over 4 lanes each instead of 16 over 2, so half the FP64
+// operations of a step and 16 warps an SM.  d = 5, k = 3, D = 4: 200 syndromes
+// 54.4 -> 34.4 ms, 1 syndrome 4.9 -> 3.6; d = 9, 60: 92.9 -> 60.2.  FP32, whose
+// rounding a change of summation order would move, keeps the one instance.
+template <typename T>
+cudaError_t launch_decode_t(const LaunchArgs& a, cudaStream_t st) {
+  if constexpr (sizeof(T) == 8) {
+    if (a.D <= 4) return launch_decode_dm<T, 4>(a, st);
+  }
+  return launch_decode_dm<T, kMaxD>(a, st);
 }
 
 template <typename T, int K>

@@ -549,30 +549,41 @@ __device__ __noinline__ void svd_step(WarpWS<T, K, DM>& ws, const Ctx<T, K>& c, 
 __device__ __forceinline__ bool pos_gt(double x, double y) { return __double_as_longlong(x) > __double_as_longlong(y); }
 __device__ __forceinline__ bool pos_lt(double x, double y) { return pos_gt(y, x); }
 
+// Sum over the 32 / R lanes that share lane mod R.
+template <int R>
+__device__ __forceinline__ double parts_sum(double v) {
+#pragma unroll
+  for (int o = R; o < 32; o <<= 1) v += __shfl_xor_sync(kFull, v, o);
+  return v;
+}
+
 // lq_step: modified Gram-Schmidt as there (two passes, the same dependence
 // test), with unnormalised rows: the products <x_i, x_j> of a step give the
-// norm of row j too, and rows are scaled once at the end of a pass.
+// norm of row j too, and rows are scaled once at the end of a pass.  A row (of
+// at most 2 DM) is spread over the warp's 32 / (2 DM) groups of lanes.
 template <int K, int DM>
 __device__ __noinline__ void lq_step64(WarpWS<double, K, DM>& ws, int s, int lane) {
-  constexpr int HC = 2 * DM;                 // places per half-row
-  static_assert(HC % 4 == 0, "places are taken four at a time");
+  constexpr int R = 2 * DM, PARTS = 32 / R;  // rows, lanes per row
+  constexpr int HC = 4 * DM / PARTS;         // places per lane
+  constexpr int CH = DM / 2;                 // places taken at a time
+  static_assert(32 % R == 0 && HC % CH == 0, "whole groups of lanes, whole groups of places");
   const int pl = ws.bond[s], pr = ws.bond[s + 1];
   const int nc = 2 * pr;                     // row length (<= 4D), even
-  const int row = lane & 15, half = lane >> 4;
+  const int row = lane & (R - 1), part = lane / R;
   const bool own = row < pl;
-  const int tb = nc >> 1;                    // places in use
+  const int tb = (nc + PARTS - 1) / PARTS;   // places in use
   double x[HC];
   const double* A = ws.psi[s];
 #pragma unroll
-  for (int t = 0; t < HC; ++t) x[t] = (own && t < tb) ? A[row * nc + 2 * t + half] : 0.0;
+  for (int t = 0; t < HC; ++t) x[t] = (own && PARTS * t + part < nc) ? A[row * nc + PARTS * t + part] : 0.0;
   double nrm0 = 0;
 #pragma unroll
-  for (int c = 0; c < HC; c += 4)
+  for (int c = 0; c < HC; c += CH)
     if (c < tb) {
 #pragma unroll
-      for (int t = c; t < c + 4; ++t) nrm0 = fma(x[t], x[t], nrm0);
+      for (int t = c; t < c + CH; ++t) nrm0 = fma(x[t], x[t], nrm0);
     }
-  nrm0 += __shfl_xor_sync(kFull, nrm0, 16);
+  nrm0 = parts_sum<R>(nrm0);
   double* L1 = ws.mat;                       // [pass][a][j] coefficients, pl x pl each
   double* L2 = ws.mat + 4 * DM * DM;
   for (int e = lane; e < 2 * 4 * DM * DM; e += 32) ws.mat[e] = 0.0;
@@ -587,15 +598,15 @@ __device__ __noinline__ void lq_step64(WarpWS<double, K, DM>& ws, int s, int lan
       if (pass == 1 && !((kept >> j) & 1u)) continue;      // zero row
       double q[HC], cf = 0;
 #pragma unroll
-      for (int c = 0; c < HC; c += 4)
+      for (int c = 0; c < HC; c += CH)
         if (c < tb) {
 #pragma unroll
-          for (int t = c; t < c + 4; ++t) {
-            q[t] = __shfl_sync(kFull, x[t], j + 16 * half);
+          for (int t = c; t < c + CH; ++t) {
+            q[t] = __shfl_sync(kFull, x[t], j + R * part);
             cf = fma(x[t], q[t], cf);
           }
         }
-      cf += __shfl_xor_sync(kFull, cf, 16);
+      cf = parts_sum<R>(cf);
       const double nj2 = __shfl_sync(kFull, cf, j);
       const bool indep = pos_gt(nj2, pass == 0 ? __shfl_sync(kFull, ref, j) : 0.0) && pos_gt(nj2, 0.0);
       if (!indep) {                          // dependent on the earlier rows: dropped, its coefficients stay
@@ -609,20 +620,20 @@ __device__ __noinline__ void lq_step64(WarpWS<double, K, DM>& ws, int s, int lan
       const double rs = inv_norm_ulp(nj2);
       const double lj = cf * rs;             // <x_row, q_j>; of row j its norm
       if (row == j) scale = rs;
-      if (own && row >= j && half == 0) Lc[row * pl + j] = lj;
+      if (own && row >= j && part == 0) Lc[row * pl + j] = lj;
       const double f = (own && row > j) ? -(lj * rs) : 0.0;
 #pragma unroll
-      for (int c = 0; c < HC; c += 4)
+      for (int c = 0; c < HC; c += CH)
         if (c < tb) {
 #pragma unroll
-          for (int t = c; t < c + 4; ++t) x[t] = fma(f, q[t], x[t]);
+          for (int t = c; t < c + CH; ++t) x[t] = fma(f, q[t], x[t]);
         }
     }
 #pragma unroll
-    for (int c = 0; c < HC; c += 4)
+    for (int c = 0; c < HC; c += CH)
       if (c < tb) {
 #pragma unroll
-        for (int t = c; t < c + 4; ++t) x[t] *= scale;
+        for (int t = c; t < c + CH; ++t) x[t] *= scale;
       }
   }
   __syncwarp();
@@ -640,7 +651,7 @@ __device__ __noinline__ void lq_step64(WarpWS<double, K, DM>& ws, int s, int lan
   if (own && ((kept >> row) & 1u)) {
 #pragma unroll
     for (int t = 0; t < HC; ++t)
-      if (t < tb) Q[myidx * nc + 2 * t + half] = x[t];
+      if (PARTS * t + part < nc) Q[myidx * nc + PARTS * t + part] = x[t];
   }
   // L = L1 * L2 restricted to kept columns: L[a][k] (pl x r) into vm (both
   // factors are lower triangular).
@@ -680,36 +691,39 @@ __device__ __noinline__ void lq_step64(WarpWS<double, K, DM>& ws, int s, int lan
 // columns are S V^T and the accumulated rotations U.
 template <int K, int DM>
 __device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<double, K>& c, int s, int lane) {
-  static_assert(DM <= 8 && DM % 4 == 0, "register Jacobi holds at most 16 columns");
+  constexpr int R = 2 * DM, PARTS = 32 / R;  // columns, lanes per column
+  constexpr int NR = 2 * DM / PARTS;         // rows per lane
+  constexpr int CH = NR / 2;                 // rows taken at a time
+  static_assert(32 % R == 0 && NR % CH == 0, "whole groups of lanes, whole groups of rows");
   const int pl = ws.bond[s], pr = ws.bond[s + 1];
   const int m = 2 * pl, n = pr;
   const bool tr = m < n;
   const int q = tr ? m : n, p = tr ? n : m;  // columns, their length
-  const int col = lane & 15, half = lane >> 4;
+  const int col = lane & (R - 1), part = lane / R;
   const bool on = col < q;
-  const int tb = (p + 1) >> 1, vb = tr ? (q + 1) >> 1 : 0;
-  double a[DM], v[DM];
+  const int tb = (p + PARTS - 1) / PARTS, vb = tr ? (q + PARTS - 1) / PARTS : 0;
+  double a[NR], v[NR];
   const double* S = ws.psi[s];
 #pragma unroll
-  for (int t = 0; t < DM; ++t) {
-    const int i = 2 * t + half;
+  for (int t = 0; t < NR; ++t) {
+    const int i = PARTS * t + part;
     a[t] = (on && i < p) ? (tr ? S[col * n + i] : S[i * n + col]) : 0.0;
     v[t] = (on && i == col) ? 1.0 : 0.0;
   }
   auto norm2 = [&]() {                       // of this lane's column
     double w = 0;
 #pragma unroll
-    for (int e = 0; e < DM; e += 4)
+    for (int e = 0; e < NR; e += CH)
       if (e < tb) {
 #pragma unroll
-        for (int t = e; t < e + 4; ++t) w = fma(a[t], a[t], w);
+        for (int t = e; t < e + CH; ++t) w = fma(a[t], a[t], w);
       }
-    return w + __shfl_xor_sync(kFull, w, 16);
+    return parts_sum<R>(w);
   };
   double own = norm2();
-  double fro = own;                          // over the 16 columns (each half holds every norm)
+  double fro = own;                          // over the columns (each group of lanes holds every norm)
 #pragma unroll
-  for (int o = 8; o > 0; o >>= 1) fro += __shfl_xor_sync(kFull, fro, o);
+  for (int o = R / 2; o > 0; o >>= 1) fro += __shfl_xor_sync(kFull, fro, o);
   const double eps = Eps<double>::v();
   const double tol2 = 16.0 * eps * eps * m;
   const double thr2 = c.cutoff2 * fro / (16.0 * n);
@@ -720,18 +734,18 @@ __device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<dou
       bool rotated = false;
       for (int rnd = 0; rnd < np - 1; ++rnd) {
         const int pj = on ? rr_partner(col, rnd, np) : col;
-        const int src = (pj & 15) | (half << 4);
-        double pa[DM], cr = 0;
+        const int src = (pj & (R - 1)) | (part * R);
+        double pa[NR], cr = 0;
 #pragma unroll
-        for (int e = 0; e < DM; e += 4)
+        for (int e = 0; e < NR; e += CH)
           if (e < tb) {
 #pragma unroll
-            for (int t = e; t < e + 4; ++t) {
+            for (int t = e; t < e + CH; ++t) {
               pa[t] = __shfl_sync(kFull, a[t], src);
               cr = fma(a[t], pa[t], cr);
             }
           }
-        cr += __shfl_xor_sync(kFull, cr, 16);
+        cr = parts_sum<R>(cr);
         const double oth = __shfl_sync(kFull, own, src);
         const bool lo = col < pj;
         const double al = lo ? own : oth, be = lo ? oth : own;
@@ -755,16 +769,16 @@ __device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<dou
           rotated = true;
         }
 #pragma unroll
-        for (int e = 0; e < DM; e += 4)
+        for (int e = 0; e < NR; e += CH)
           if (e < tb) {
 #pragma unroll
-            for (int t = e; t < e + 4; ++t) a[t] = fma(sn, pa[t], cs * a[t]);
+            for (int t = e; t < e + CH; ++t) a[t] = fma(sn, pa[t], cs * a[t]);
           }
 #pragma unroll
-        for (int e = 0; e < DM; e += 4)
+        for (int e = 0; e < NR; e += CH)
           if (e < vb) {
 #pragma unroll
-            for (int t = e; t < e + 4; ++t) v[t] = fma(sn, __shfl_sync(kFull, v[t], src), cs * v[t]);
+            for (int t = e; t < e + CH; ++t) v[t] = fma(sn, __shfl_sync(kFull, v[t], src), cs * v[t]);
           }
         own = norm2();
       }
@@ -781,7 +795,7 @@ __device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<dou
     smax = si > smax ? si : smax;
   }
   const double floor2 = c.cutoff2 * smax > noise2 ? c.cutoff2 * smax : noise2;
-  const int keep = __popc(__ballot_sync(kFull, half == 0 && sq > floor2));
+  const int keep = __popc(__ballot_sync(kFull, part == 0 && sq > floor2));
   int r = imin(imin(keep, c.D), m);
   if (r < 1) r = 1;
   __syncwarp();
@@ -791,8 +805,8 @@ __device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<dou
   if (on && rank < r) {
     const double inv = tr ? 1.0 : inv_norm_ulp(sq);
 #pragma unroll
-    for (int t = 0; t < DM; ++t) {
-      const int i = 2 * t + half;
+    for (int t = 0; t < NR; ++t) {
+      const int i = PARTS * t + part;
       if (tr) {
         if (i < n) svt[rank * n + i] = a[t];
         if (i < m) U[i * r + rank] = v[t];

@@ -28,3 +28,17 @@ def test_outputs_do_not_depend_on_the_cluster_size(precision, d, k, D, sizes):
         for key in ("logp", "delta", "iters", "flags", "decision"):
             assert torch.equal(out[key], outs[-1][key][:n]), (n, key)
             assert torch.equal(out[key], again[key]), (n, key)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("k,d,B", [(1, 3, 5), (1, 4, 40), (2, 2, 3), (2, 3, 300), (2, 4, 1), (2, 5, 30), (2, 7, 9)])
+def test_small_bond_instance_equals_the_fused_form(k, d, B):
+    # k <= 2 and D = 4 truncate nothing, so the instance for D <= 4 gives the
+    # fused form's log P (FP64 bar 1e-9) and, iteration by iteration, its stops.
+    _, _, S = synth.sample_syndromes(7900 + d, 0, B, d, 0.1)
+    S = torch.from_numpy(S).cuda()
+    prm = dict(d=d, k=k, D=4, p=0.1, max_iter=6, delta0=0.0, precision="fp64")
+    a = pkg.decode(S, pkg.DecoderParams(algorithm="mps", **prm))
+    b = pkg.decode(S, pkg.DecoderParams(algorithm="fused", **prm))
+    assert torch.equal(a["iters"], b["iters"])
+    assert float((a["logp"] - b["logp"]).abs().max()) <= 1e-9
