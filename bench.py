@@ -114,14 +114,15 @@ def run_oracle_sample(first_shot: int, n: int, procs: int, algorithm: str):
     return dt, res
 
 
-# Multiply-adds of the 4 x 4 register form per (row, coset): column 0's two
-# butterflies 6; per upper leg a0 of column 0 (two): column 1's upper-qubit
-# butterflies 4 and lower-qubit products 4, the upper side message's
-# entries 4, column 2's butterflies and data column 16; the lower side
-# message's data column 8; column 3 6.  Only the entries with column 3's
-# upper leg e equal to the row's bit r0 (the check at its top ties them)
-# are formed.
-REGISTER_FORM_MADDS = 76
+# Multiply-adds of the 4 x 4 register form per (row, coset): the upper side
+# message's table 2 (8 per pair of rows' legs, shared by four rows); column 0's
+# two butterflies 6; per upper leg a0 of column 0 (two): column 1's upper-qubit
+# butterfly 2, then for the lower leg its qubit does not tell apart and for
+# each of the two it does (three): the lower qubit's factor 1, column 2's lower
+# butterfly 2 and its data column 2; the lower side message's data column 8;
+# column 3 6.  Only the entries with column 3's upper leg e equal to the row's
+# bit r0 (the check at its top ties them) are formed.
+REGISTER_FORM_MADDS = 56
 
 
 def fused_flops(d: int, k: int):
@@ -190,7 +191,7 @@ def fused_flops(d: int, k: int):
                 if h == 4 and len(lines) == 4:
                     # 4 x 4 blocks: the register form of the update (butterflies
                     # over single row bits, side messages contracted where their
-                    # legs enter), 76 multiply-adds per (row, coset) entry
+                    # legs enter), 56 multiply-adds per (row, coset) entry
                     # whichever node column 0 starts with (a chain starting with
                     # a check is read bottom to top).
                     per_iter += 2.0 * 16 * REGISTER_FORM_MADDS + 12.0 * 2 ** h
@@ -292,10 +293,10 @@ def mixed_batch_leg(args, dev, pkg):
     packed, offsets, d_of = pack_mixed(shots, device=dev)
     prm = pkg.DecoderParams(d=0, k=K_BLOCK, p=P_NOISE, max_iter=MAX_ITER, eta=ETA, delta0=DELTA0, delta1=DELTA1,
                             precision="fp32", algorithm="fused")
-    # Every distance here is odd, so the register-form-only kernels are candidates too.
+    # The default kernel first; every distance here is odd, so the register-form-only kernels are candidates too.
     lean = ((8, 4, 3), (8, 2, 3)) if all(d % 2 == 1 for d in MIXED_DISTANCES) else ()
     prm, table = autotune.tune_mixed(packed, offsets, d_of, prm,
-                                     shapes=lean + ((8, 4, 1), (8, 4, 2), (8, 2, 1), (8, 2, 2), (4, 2, 1), (4, 4, 1)),
+                                     shapes=((0, 0, 0),) + lean + ((8, 4, 1), (8, 4, 2), (8, 2, 1), (8, 2, 2), (4, 2, 1), (4, 4, 1)),
                                      ctas=(0, 1, 2))
     order = torch.argsort(d_of, descending=True, stable=True).to(torch.int32)
     d_max = int(max(MIXED_DISTANCES))
@@ -351,7 +352,7 @@ def mixed_batch_leg(args, dev, pkg):
             "counts": [int(c) for c in counts], "p": P_NOISE, "precision": "fp32", "algorithm": "fused",
             "launch": "one persistent launch, largest distance first, replayed from a CUDA graph",
             "shape": {"warps": prm.warps, "cosets": prm.cosets,
-                      "messages": {1: "shared", 2: "workspace", 3: "shared, register form only"}[prm.messages],
+                      "messages": {0: "default", 1: "shared", 2: "workspace", 3: "shared, register form only"}[prm.messages],
                       "ctas_per_sm": prm.ctas_per_sm},
             "autotune_candidates": len(table),
             "mean_iters": float(out["iters"].double().mean().item()),
@@ -633,7 +634,7 @@ def ours(args):
                 "launch_ms": dec_ms,
                 "peak_source": (f"derived: {per_clk} {'FP32 lanes' if fp else 'FP64 FMA/clk'} per SM x 2 x "
                                 f"{n_sm} SMs x {sm_mhz:.0f} MHz (max SM clock)"),
-                "flop_model": "4x4 blocks: the multiply-adds of the register form (76 per row and "
+                "flop_model": "4x4 blocks: the multiply-adds of the register form (56 per row and "
                               "coset); other blocks: qubit nodes as 2x2 XOR convolutions (4 multiply-adds "
                               "per state entry), check nodes as zero-flop copy tensors, side-message data "
                               "columns; normalise/damp/overlap; Lemma 1 read-out (register form for 4x4 blocks)",

@@ -104,9 +104,10 @@ extern "C" {
  *             3 shared memory with every block update in register form:
  *             k = 4 at odd d only, where every block is 4 x 4 or one node
  *             wide; small per-warp buffers, sized for more CTAs per SM; for
- *             bbp_decode_mixed only on request, see there).
- *             0 picks by geometry and, for FP32 at k = 4 and odd d, by batch
- *             size (few syndromes: one coset per CTA); where the geometry's
+ *             bbp_decode_mixed see there).
+ *             0 picks the kernel by geometry, precision and batch size (few
+ *             syndromes: one coset per CTA; k = 4 at any d and k = 5, 6 have
+ *             kernels that only the default reaches); where the geometry's
  *             messages do not fit in shared memory, workspace slots;
  *             compiled (warps, cosets):
  *             FP32 (8,4) (8,2) (4,2) (4,4) (16,1) (8,1) (4,1), of which (8,4)
@@ -460,7 +461,7 @@ int bbp_decode_warm_workspace_bytes(const bbp_params* prm, int64_t B, int includ
  *              the register-form-only kernels: the caller vouches that every
  *              distance is odd (k = 4, d_max odd, else BBP_EUNSUPPORTED); a
  *              syndrome of even distance in such a batch gets
- *              BBP_FLAG_CAPACITY.  The default never takes them.
+ *              BBP_FLAG_CAPACITY.  The default holds for every distance.
  *   workspace  device, at least 256 bytes (the work counter); when the launch
  *              shape keeps its messages in the workspace (always for k = 5,
  *              6), 256 + bbp_workspace_bytes of d_max and B (the slots)

@@ -35,15 +35,17 @@ def _time(fn, reps=3):
 
 
 def candidates(prm: DecoderParams):
-    """Compiled (warps, cosets, messages) of the fused kernel: messages 1 in
-    shared memory, 2 in workspace slots (always for k = 5, 6), 3 every block
-    update in register form (k = 4 at odd d)."""
+    """(warps, cosets, messages) of the fused kernel: (0, 0, 0) is the default,
+    which picks its kernel by geometry and batch and has kernels of its own;
+    then the compiled shapes, messages 1 in shared memory, 2 in workspace
+    slots (always for k = 5, 6), 3 every block update in register form (k = 4
+    at odd d)."""
     if prm.k > 4:
-        return tuple((w, c, 2) for w, c in FUSED_SHAPES_K6[prm.precision])
+        return ((0, 0, 0),) + tuple((w, c, 2) for w, c in FUSED_SHAPES_K6[prm.precision])
     lean = ()
     if prm.k == 4 and prm.d % 2 == 1:
         lean = tuple((w, c, 3) for w, c in FUSED_SHAPES_LEAN[prm.precision])
-    return (lean + tuple((w, c, 1) for w, c in FUSED_SHAPES[prm.precision]) +
+    return (((0, 0, 0),) + lean + tuple((w, c, 1) for w, c in FUSED_SHAPES[prm.precision]) +
             tuple((w, c, 2) for w, c in FUSED_SHAPES_WS[prm.precision]))
 
 
