@@ -1337,16 +1337,19 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
       }
       cluster_barrier();
       if (tid == 0) misc[0] = 0;   // only rank 0's counts
+      // Remark 4: Delta = sqrt(sum_i 2 - 2 <m_i^t | m_i^(t-1)>^2) / M.  Every
+      // CTA sums its own copy of the overlaps between the two barriers: the
+      // first orders the peers' stores of this iteration before the sum, the
+      // second the sum before those of the next, so all CTAs hold the same
+      // Delta and leave the loop together.
+      if (color == 1 && warp == 0) {
+        double acc = 0.0;
+        for (int i = lane; i < M; i += 32) acc += 2.0 - 2.0 * ovl[i] * ovl[i];
+        acc = warp_sum(acc);
+        if (lane == 0) dsh[0] = sqrt(fmax(acc, 0.0)) / M;
+      }
       cluster_barrier();
     }
-    // Remark 4: Delta = sqrt(sum_i 2 - 2 <m_i^t | m_i^(t-1)>^2) / M.
-    if (warp == 0) {
-      double acc = 0.0;
-      for (int i = lane; i < M; i += 32) acc += 2.0 - 2.0 * ovl[i] * ovl[i];
-      acc = warp_sum(acc);
-      if (lane == 0) dsh[0] = M > 0 ? sqrt(fmax(acc, 0.0)) / M : 0.0;
-    }
-    __syncthreads();
     delta = dsh[0];
     it_done = it;
     if (delta < a.delta0) break;
