@@ -22,6 +22,7 @@
 #include <stdint.h>
 
 #include "bbp_geometry.h"
+#include "bbp_jacobi.h"
 
 namespace bbp {
 
@@ -549,6 +550,13 @@ __device__ __noinline__ void svd_step(WarpWS<T, K, DM>& ws, const Ctx<T, K>& c, 
 __device__ __forceinline__ bool pos_gt(double x, double y) { return __double_as_longlong(x) > __double_as_longlong(y); }
 __device__ __forceinline__ bool pos_lt(double x, double y) { return pos_gt(y, x); }
 
+// x 2^(ex / 2^20) for ex a multiple of 2^20 and a result below 2^1024, on the
+// exponent bits; a result below the normal range is 0.
+__device__ __forceinline__ double exp_add(double x, int ex) {
+  const int hi = __double2hiint(x), e = hi & 0x7ff00000;
+  return e > 0 && e + ex > 0 ? __hiloint2double(hi + ex, __double2loint(x)) : 0.0;
+}
+
 // Sum over the 32 / R lanes that share lane mod R.
 template <int R>
 __device__ __forceinline__ double parts_sum(double v) {
@@ -684,11 +692,10 @@ __device__ __noinline__ void lq_step64(WarpWS<double, K, DM>& ws, int s, int lan
 // svd_step: one-sided Jacobi on the site matrix A (m x n) or, when m < n, on
 // its transpose, so that the q = min(m, n) columns it rotates are the fewer
 // (site 0 has m = 2 rows per left bond).  A pair's rotation solves c t^2 + (b
-// - a) t - c = 0 (a, b the squared norms, c the product) by an FP32 root and
-// one Newton step whose residual is FP64; the cosine is an exact unit-norm
-// scale of that t, so the rotation is orthogonal to rounding whatever t's
-// last bits are.  m >= n: U are the scaled columns, S V^T = U^T A.  m < n: the
-// columns are S V^T and the accumulated rotations U.
+// - a) t - c = 0 (a, b the squared norms, c the product) to two FP64 roundings
+// (jacobi_tangent), and the cosine is the unit-norm scale of that t.  m >= n: U
+// are the scaled columns, S V^T = U^T A.  m < n: the columns are S V^T and the
+// accumulated rotations U.
 template <int K, int DM>
 __device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<double, K>& c, int s, int lane) {
   constexpr int R = 2 * DM, PARTS = 32 / R;  // columns, lanes per column
@@ -755,15 +762,9 @@ __device__ __noinline__ void svd_step64(WarpWS<double, K, DM>& ws, const Ctx<dou
         if (!__any_sync(kFull, rot)) continue;
         double cs = 1.0, sn = 0.0;
         if (rot) {
-          // Scaled by a power of two so that FP32 holds them.
+          // Scaled by a power of two (on the exponent bits) so that FP32 holds them.
           const int ex = (1023 << 20) - (max(__double2hiint(al), __double2hiint(be)) & 0x7ff00000);
-          const double sc = __hiloint2double((1023 << 20) + max(-(1000 << 20), min(1000 << 20, ex)), 0);
-          const double d = (be - al) * sc, cc = cr * sc;
-          const float df = (float)d, cf = (float)cc, z = df / (2.f * cf), az = fabsf(z);
-          const float tf = copysignf(az > 1e4f ? 0.5f / az : 1.f / (az + sqrtf(fmaf(az, az, 1.f))), z);
-          const double t0 = (double)tf;
-          const double res = fma(fma(cc, t0, d), t0, -cc);
-          const double t1 = t0 - (double)((float)res / fmaf(2.f * cf, tf, df));
+          const double t1 = jacobi_tangent(exp_add(be - al, ex), exp_add(cr, ex));
           cs = rsqrt_unit(fma(t1, t1, 1.0));
           sn = lo ? -(cs * t1) : cs * t1;
           rotated = true;
