@@ -64,15 +64,21 @@ struct FusedWS {   // (sizes for block side K: slot = FusedDim<K>::slot, vec = F
 // full blocks node by node, takes full-size buffers from the same memory with
 // fewer warps.
 template <int K>
-BBP_HD int fused_slot(const Geo& g, int lean) {
-  if (K <= 4 || !lean) return FusedDim<K>::slot;
-  return g.k == 6 && g.W % 6 == 5 ? 2 * kBlock6Buf : kBlock6Buf;   // a 6 x 5 block's widest state has 2^11 entries
+BBP_HD int fused_slot(int lean) {
+  return K <= 4 || !lean ? FusedDim<K>::slot : kBlock6Buf;
 }
 
+// Geometries whose block states at k = 5, 6 fit the small buffers: all but
+// those with 6 x 5 blocks, whose widest state has 2^11 entries (k = 6 and d a
+// multiple of 3).  With buffers of that size at most 8 FP32 warps, and fewer
+// than 8 in FP64, would fit an SM; these distances take the kernels with
+// full-size buffers (6 warps, 3 in FP64).
+BBP_HD bool small_states(const Geo& g) { return g.k == 5 || (g.k == 6 && g.W % 6 != 5); }
+
 template <typename T, int K>
-BBP_HD int fused_ws_bytes(const Geo& g, int G, int lean = 0) {
+BBP_HD int fused_ws_bytes(int G, int lean = 0) {
   if (K == 4 && lean) return align_up((int)sizeof(T) * kRegStage, 16);
-  return align_up((int)sizeof(T) * G * (2 * fused_slot<K>(g, lean) + 16 + 2 * FusedDim<K>::vec), 16);
+  return align_up((int)sizeof(T) * G * (2 * fused_slot<K>(lean) + 16 + 2 * FusedDim<K>::vec), 16);
 }
 
 template <typename T, int K>
@@ -134,9 +140,9 @@ BBP_HD FusedLayout fused_layout(const Geo& g, int M, int nwarps, int G, bool gm 
   L.msgs = o;   // the messages, unless they live in the workspace
   if (!gm) o = align_up(o + (int)sizeof(T) * G * fused_coset_stride<K>(M, gm), 16);
   L.ws = o;
-  L.ws_stride = fused_ws_bytes<T, K>(g, G, lean);
+  L.ws_stride = fused_ws_bytes<T, K>(G, lean);
   int ws = nwarps * L.ws_stride;
-  if (K == 4 && lean == 2) ws = imax(ws, kReadWarps * fused_ws_bytes<T, K>(g, 1));
+  if (K == 4 && lean == 2) ws = imax(ws, kReadWarps * fused_ws_bytes<T, K>(1));
   o = align_up(o + ws, 16);
   L.total = o;
   return L;
@@ -1146,7 +1152,7 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   c.frame = frames; c.msg_of = msg_of; c.msg_off = nullptr; c.dims = nullptr;
   c.arena = nullptr; c.e0 = nullptr; c.cta_flags = &misc[4];
   FusedWS<T> ws{};
-  if constexpr (!kLean) ws = fused_ws_at<T, K>(smem + Lo.ws + warp * Lo.ws_stride, G, fused_slot<K>(g, kMode));
+  if constexpr (!kLean) ws = fused_ws_at<T, K>(smem + Lo.ws + warp * Lo.ws_stride, G, fused_slot<K>(kMode));
 
   const T pI = a.pI_w, pE = a.pE_w;
   const RegUpd<T> upd{a.eta_w, a.one_m_eta_w, ovl, M};
@@ -1328,7 +1334,7 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
     // warp's buffers are in use any more but the passes' above.
     const int nf = W / 4, cnt = W % 4 == 3 ? 2 * nf + 1 : 0;
     __syncthreads();
-    ws = fused_ws_at<T, K>(smem + Lo.ws + (warp < kReadWarps ? warp : 0) * fused_ws_bytes<T, K>(g, 1), 1,
+    ws = fused_ws_at<T, K>(smem + Lo.ws + (warp < kReadWarps ? warp : 0) * fused_ws_bytes<T, K>(1), 1,
                            FusedDim<K>::slot);
     for (int j = warp; warp < kReadWarps && j < cnt * G; j += kReadWarps) {
       const int i = j / G, q = j % G;
@@ -1347,7 +1353,7 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   if constexpr (!kLean) {
     const unsigned all = G == 1 ? 0u : (G == 2 ? 0x4u : 0xE4u);    // slot q holds coset q
     c.frame = frames;
-    const int full = fused_ws_bytes<T, K>(g, G);                   // full-size state buffers
+    const int full = fused_ws_bytes<T, K>(G);                   // full-size state buffers
     const int nro = K > 4 && LB > 0 ? imin(NW, NW * Lo.ws_stride / full) : NW;
     if (K > 4 && LB > 0 && warp < nro)
       ws = fused_ws_at<T, K>(smem + Lo.ws + warp * full, G, FusedDim<K>::slot);

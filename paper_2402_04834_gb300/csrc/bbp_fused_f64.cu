@@ -167,10 +167,12 @@ bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, in
 // codes ((4, 4, 3) at d = 5, 1000 syndromes: a quarter less than (8, 2, 2));
 // small batches gain most (one syndrome at d = 11: (16, 1) 0.58 of (4, 2)).
 // Block sides 5 and 6 (messages in workspace slots, one coset per CTA): the
-// kernels with small state buffers, 16 warps per SM (8 in FP64).
+// kernels with small state buffers, 16 warps per SM (8 in FP64), where every
+// block's state fits them (not at k = 6 and d a multiple of 3: small_states).
 bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, bool odd, int* warps, int* cosets,
                 int* lean) {
   if (g.k > 4) {
+    if (!small_states(g)) return false;
     auto fit6 = [&](int w) {
       const int smem = precision == 0 ? fused_smem_for<double, 6>(g, M, w, 1, true, true)
                                       : fused_smem_for<float, 6>(g, M, w, 1, true, true);
