@@ -4,8 +4,9 @@ The results never depend on the launch shape; only the time does.  For a
 given workload the tuner times every candidate (warps per CTA, cosets per
 CTA, messages in shared memory or in workspace slots, and for mixed batches
 resident CTAs per SM) with CUDA events and
-keeps the fastest, caching the choice per workload signature for the life
-of the process.  Shapes whose shared memory does not fit are skipped.
+keeps the fastest, caching the choice per workload signature (batch sizes by
+powers of two: a shape that fills the chip with a long batch is a slow one for
+a few syndromes) for the life of the process.  Shapes whose shared memory does not fit are skipped.
 """
 
 from __future__ import annotations
@@ -52,7 +53,7 @@ def candidates(prm: DecoderParams):
 def tune_uniform(syndromes, prm: DecoderParams, shapes=None):
     """Best (warps, cosets, messages) for a same-distance batch; returns (params, table)."""
     shapes = tuple(shapes or candidates(prm))
-    key = ("uniform", prm.d, prm.k, prm.precision, prm.max_iter, shapes)
+    key = ("uniform", prm.d, int(syndromes.shape[0]).bit_length(), prm.k, prm.precision, prm.max_iter, shapes)
     if key in _cache:
         return dataclasses.replace(prm, **_cache[key][0]), _cache[key][1]
     table = []
@@ -78,7 +79,7 @@ def tune_mixed(packed, offsets, d_of, prm: DecoderParams, shapes=None, ctas=(0, 
         if prm.k == 4 and all(d % 2 == 1 for d in sig):
             shapes = tuple((w, c, 3) for w, c in FUSED_SHAPES_LEAN[prm.precision]) + tuple(shapes)
     shapes = tuple(shapes)
-    key = ("mixed", sig, prm.k, prm.precision, prm.max_iter, shapes, tuple(ctas))
+    key = ("mixed", sig, int(d_of.shape[0]).bit_length(), prm.k, prm.precision, prm.max_iter, shapes, tuple(ctas))
     if key in _cache:
         return dataclasses.replace(prm, **_cache[key][0]), _cache[key][1]
     table = []
