@@ -75,7 +75,7 @@ def tune_mixed(packed, offsets, d_of, prm: DecoderParams, shapes=None, ctas=(0, 
     distance of the batch is odd (k = 4)."""
     sig = tuple(sorted(torch.unique(d_of).tolist()))
     if shapes is None:
-        shapes = candidates(prm)
+        shapes = candidates(dataclasses.replace(prm, d=0))     # the batch decides, not prm.d
         if prm.k == 4 and all(d % 2 == 1 for d in sig):
             shapes = tuple((w, c, 3) for w, c in FUSED_SHAPES_LEAN[prm.precision]) + tuple(shapes)
     shapes = tuple(shapes)

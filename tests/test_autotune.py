@@ -40,3 +40,16 @@ def test_a_shape_is_not_carried_over_to_another_batch_size(timed):
         before = len(timed)
         autotune.tune_mixed(None, None, torch.tensor([7, 9] * (B // 2), dtype=torch.int32), odd, ctas=(0,))
         assert (len(timed) > before) == again, B
+
+
+def test_register_form_only_shapes_need_a_batch_of_odd_distances(timed):
+    # decode_mixed takes messages = 3 as the caller's word that every distance
+    # is odd and flags a syndrome of even distance; prm.d says nothing about it.
+    for d in (0, 11):
+        prm = pkg.DecoderParams(d=d, k=4, precision="fp32", algorithm="fused")
+        for ds, lean in (([8, 11], False), ([7, 11], True)):
+            del timed[:]
+            autotune._cache.clear()
+            autotune.tune_mixed(None, None, torch.tensor(ds, dtype=torch.int32), prm, ctas=(0,))
+            assert any(shape[2] == 3 for _, shape in timed) == lean, (d, ds)
+            assert len(timed) == len(set(timed))
