@@ -293,8 +293,9 @@ def mixed_batch_leg(args, dev, pkg):
     packed, offsets, d_of = pack_mixed(shots, device=dev)
     prm = pkg.DecoderParams(d=0, k=K_BLOCK, p=P_NOISE, max_iter=MAX_ITER, eta=ETA, delta0=DELTA0, delta1=DELTA1,
                             precision="fp32", algorithm="fused")
-    # The default kernel first; every distance here is odd, so the register-form-only kernels are candidates too.
-    lean = ((8, 4, 3), (8, 2, 3)) if all(d % 2 == 1 for d in MIXED_DISTANCES) else ()
+    # The default kernel first; every distance here is odd, so the register-form-only kernels are candidates too
+    # ((0, 0, 3): those the default picks from).
+    lean = ((0, 0, 3), (8, 4, 3), (8, 2, 3)) if all(d % 2 == 1 for d in MIXED_DISTANCES) else ()
     prm, table = autotune.tune_mixed(packed, offsets, d_of, prm,
                                      shapes=((0, 0, 0),) + lean + ((8, 4, 1), (8, 4, 2), (8, 2, 1), (8, 2, 2), (4, 2, 1), (4, 4, 1)),
                                      ctas=(0, 1, 2))

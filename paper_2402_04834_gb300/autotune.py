@@ -77,7 +77,8 @@ def tune_mixed(packed, offsets, d_of, prm: DecoderParams, shapes=None, ctas=(0, 
     if shapes is None:
         shapes = candidates(dataclasses.replace(prm, d=0))     # the batch decides, not prm.d
         if prm.k == 4 and all(d % 2 == 1 for d in sig):
-            shapes = tuple((w, c, 3) for w, c in FUSED_SHAPES_LEAN[prm.precision]) + tuple(shapes)
+            # (0, 0, 3): the default's own register-form-only kernels.
+            shapes = ((0, 0, 3),) + tuple((w, c, 3) for w, c in FUSED_SHAPES_LEAN[prm.precision]) + tuple(shapes)
     shapes = tuple(shapes)
     key = ("mixed", sig, int(d_of.shape[0]).bit_length(), prm.k, prm.precision, prm.max_iter, shapes, tuple(ctas))
     if key in _cache:

@@ -52,4 +52,5 @@ def test_register_form_only_shapes_need_a_batch_of_odd_distances(timed):
             autotune._cache.clear()
             autotune.tune_mixed(None, None, torch.tensor(ds, dtype=torch.int32), prm, ctas=(0,))
             assert any(shape[2] == 3 for _, shape in timed) == lean, (d, ds)
+            assert ((2, (0, 0, 3)) in timed) == lean                # the default's choice among them
             assert len(timed) == len(set(timed))
