@@ -1022,7 +1022,7 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
   // Message table in (I, J, dir) order, and each message's rank in its class.
   const int NK = nb * nb * 4;
   auto class_of = [&](int I, int J, int dir) {
-    int c = kClassNone + (dir & 1);                   // one direction's code at a time: k = 6 blocks have two forms
+    int c = kClassNone + (K > 4 ? dir & 1 : 0);       // one direction's code at a time: k = 6 blocks have two forms
     if (reg) {
       const RegFrame f = reg_frame(g, I, J, dir);
       const int sh = f.shape();
