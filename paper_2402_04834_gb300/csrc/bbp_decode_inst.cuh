@@ -102,6 +102,19 @@ int fused_smem_for(const Geo& g, int M, int warps, int cosets, bool gm = (K > 4)
   return fused_layout<T, K>(g, M, warps, cosets, gm, lean).total;
 }
 
+// Dynamic shared memory of a launch with its messages in workspace slots.  They
+// are read through L1, which gets what shared memory leaves, and the runtime
+// sets shared memory aside for every CTA that could be resident: with one CTA
+// per SM to run, room for a second takes that much from L1, so the request is
+// raised until a second would not fit (where two would leave less).  FP32, up to
+// 152 CTAs, without -> with: k = 2, 60 syndromes at d = 25 19.6 -> 14.0 ms and at
+// d = 13 5.66 -> 4.05 ms; k = 3 at d = 18 7.66 -> 6.11 ms.  With more CTAs than
+// SMs a second one pays (d = 25, 150 syndromes 26.0 ms, alone on its SM 27.9).
+inline int slot_smem(int smem, long long items, int sms) {
+  const int one = kSmemPerSm / 2;
+  return items <= sms && smem < one && 2 * (smem + kSmemReservedPerCta) > one ? one : smem;
+}
+
 template <typename T>
 KArgs<T> fused_args(const LaunchArgs& a) {
   KArgs<T> k;
@@ -115,20 +128,23 @@ KArgs<T> fused_args(const LaunchArgs& a) {
   return k;
 }
 
+inline cudaError_t sm_count(int* sms) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  return e != cudaSuccess ? e : cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
+}
+
 // Persistent grid of a launch with its messages in workspace slots:
 // resident CTAs, at most one per item and per message slot.
 template <typename Kern>
-cudaError_t persistent_grid(Kern kern, int threads, int smem, int ctas_per_sm, long long items, long long slots,
-                            long long* grid) {
+cudaError_t persistent_grid(Kern kern, int threads, int smem, int ctas_per_sm, int sms, long long items,
+                            long long slots, long long* grid) {
   cudaError_t e;
   int per_sm = ctas_per_sm;
   if (per_sm <= 0) {
     if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem)) != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
   }
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   long long g = (long long)sms * per_sm;
   if (g > items) g = items;
   if (g > slots) g = slots;
@@ -141,18 +157,23 @@ cudaError_t persistent_grid(Kern kern, int threads, int smem, int ctas_per_sm, l
 template <typename T, int NW, int G, int K, bool GM = (K > 4), int LB = 0>
 cudaError_t launch_fused_nw(const LaunchArgs& a, cudaStream_t st) {
   const KArgs<T> k = fused_args<T>(a);
-  const int smem = fused_smem_for<T, K>(a.geo, a.M, NW, G, GM, LB == 0 ? 0 : (K == 4 && LB >= kEvenLB ? 2 : 1));
+  int smem = fused_smem_for<T, K>(a.geo, a.M, NW, G, GM, LB == 0 ? 0 : (K == 4 && LB >= kEvenLB ? 2 : 1));
   auto kern = fused_kernel<T, NW, G, K, GM, LB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-  if (e != cudaSuccess) return e;
   const long long items = a.B * (4 / G);
+  int sms = 0;
+  cudaError_t e;
+  if (GM) {
+    if ((e = sm_count(&sms)) != cudaSuccess) return e;
+    smem = slot_smem(smem, items, sms);
+  }
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
   if (GM) {
     KArgs<T> kp = k;
     kp.arena = static_cast<T*>(a.arena);
     kp.n_items = items;
     kp.slot_elems = (long long)G * a.M * FusedDim<K>::vec;
     long long grid = 0;
-    if ((e = persistent_grid(kern, NW * 32, smem, 0, items, a.slots, &grid)) != cudaSuccess) return e;
+    if ((e = persistent_grid(kern, NW * 32, smem, 0, sms, items, a.slots, &grid)) != cudaSuccess) return e;
     kern<<<(unsigned)grid, NW * 32, smem, st>>>(kp);
     return cudaGetLastError();
   }
@@ -166,19 +187,19 @@ cudaError_t launch_fused_mixed_nw(const LaunchArgs& a, const MixedLaunch& m, cud
   const Geo gmax = make_geo(m.d_max, a.geo.k);
   int Mmax = 0, ae = 0;
   count_messages(gmax, 1, &Mmax, &ae);
-  const int smem = fused_smem_for<T, K>(gmax, Mmax, NW, G, GM, LB == 0 ? 0 : (K == 4 && LB >= kEvenLB ? 2 : 1));
+  int smem = fused_smem_for<T, K>(gmax, Mmax, NW, G, GM, LB == 0 ? 0 : (K == 4 && LB >= kEvenLB ? 2 : 1));
   auto kern = fused_mixed_kernel<T, NW, G, K, GM, LB>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  int sms = 0;
+  cudaError_t e = sm_count(&sms);
   if (e != cudaSuccess) return e;
+  if (GM) smem = slot_smem(smem, a.B * (4 / G), sms);
+  if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) != cudaSuccess) return e;
   int per_sm = m.ctas_per_sm;
   if (per_sm <= 0) {
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, NW * 32, smem);
     if (e != cudaSuccess) return e;
     if (per_sm < 1) per_sm = 1;
   }
-  int dev = 0, sms = 0;
-  if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
-  if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   MixedArgs mx;
   mx.d_of = m.d_of; mx.offsets = m.offsets; mx.order = m.order; mx.counter = m.counter;
   mx.n_items = a.B * (4 / G); mx.k = a.geo.k;
