@@ -169,6 +169,10 @@ bool fused_shape(int precision, const Geo& g, int M, int* warps, int* cosets, in
 // Block sides 5 and 6 (messages in workspace slots, one coset per CTA): the
 // kernels with small state buffers, 16 warps per SM (8 in FP64), where every
 // block's state fits them (not at k = 6 and d a multiple of 3: small_states).
+// In FP32 a half-round of at most six messages (two blocks a side), one network
+// per SM, is no more than the full-size kernel's six warps, which have twice the
+// registers: k = 5, d = 5, 30 syndromes 230 us against 256 (d = 6, 12 messages: 393
+// against 319), k = 6, d = 5: 194 against 227.
 bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, bool odd, int* warps, int* cosets,
                 int* lean) {
   if (g.k > 4) {
@@ -188,6 +192,7 @@ bool fused_pick(int precision, const Geo& g, int M, long long B, int sms, bool o
       *warps = 8; *lean = 2;
       return true;
     }
+    if (4 * B <= sms && (M + 1) / 2 <= 6) return false;
     if (fit6(16) < 1) return false;
     *warps = 16; *lean = 1;
     return true;
