@@ -12,7 +12,7 @@ int smem_bytes_for(const Geo& g, int M, int warps = kWarps) {
   return cta_layout(g, M, kMaxK, warps, (int)sizeof(WarpWS<T, kMaxK, DM>)).total;
 }
 
-template <typename T, int DM, int NW>
+template <typename T, int DM, int NW, bool CL>
 cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) {
   KArgs<T> k;
   k.geo = a.geo; k.M = a.M; k.D = a.D; k.max_iter = a.max_iter; k.arena_elems = a.arena_elems;
@@ -23,7 +23,7 @@ cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) 
   k.n_items = 0; k.slot_elems = 0;
   set_working(k);
   const int smem = smem_bytes_for<T, DM>(a.geo, a.M, NW);
-  auto kern = decode_kernel<T, kMaxK, DM, NW>;
+  auto kern = decode_kernel<T, kMaxK, DM, NW, CL>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
   if (e != cudaSuccess) return e;
   cudaLaunchAttribute at[1];
@@ -43,15 +43,20 @@ cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) 
 // Warps per CTA (one message update each) and CTAs per network.  The linear
 // algebra is a chain of short dependent steps, and one SM holds 8 warps in FP64
 // and 16 in FP32 (the warps' shared memory; 16 in FP64 with DM = 4 by the
-// registers), so what a batch leaves idle goes
-// to clusters that share a network's half-round (60 updates at d = 11, 12 at
-// d = 5 with k = 3), up to a warp per update:
+// registers), so what a batch leaves idle goes to clusters that share a
+// network's half-round (60 updates at d = 11, 12 at d = 5 with k = 3), up to a
+// warp per update:
 // - FP64: four-warp CTAs, as many per network as are resident together, from
 //   three on; eight-warp CTAs where even those leave half the chip idle; else
-//   pairs of eight-warp CTAs (shorter rounds, a fuller last wave).
+//   pairs of eight-warp CTAs at any batch size (shorter rounds, a fuller last
+//   wave).  Half-rounds of fewer than 16 updates: four-warp CTAs, a warp per
+//   update (d = 5, k = 3, 200 syndromes: 3 x 4 warps 54.5 ms, 1 x 8 56.0, 2 x 8
+//   67.6).
 // - FP32: eight-warp CTAs, as many per network as are resident, at least two.
-// - Half-rounds of fewer than 16 updates: four-warp CTAs, a warp per update (d =
-//   5, k = 3, 200 syndromes: 3 x 4 warps 54.5 ms, 1 x 8 56.0, 2 x 8 67.6).
+//   Half-rounds of fewer than 16 updates, whose warps the edge blocks leave
+//   idle, and k = 1, where an update is shorter than what a cluster adds to it,
+//   are shared only as far as CTAs are resident (d = 5, 150 syndromes: 1 x 4 9.4
+//   ms, 3 x 4 11.9; k = 1, d = 9, 76 syndromes: 1 x 8 7.7 ms, 2 x 8 8.8).
 // ms, one CTA per network -> clusters: FP64 d = 11, 1 syndrome 223 -> 40 (8 x 8
 // warps; 8 x 4: 49), 5: 223 -> 59 (8 x 4; 8 x 8: 63), 12: 224 -> 84, 24: 225 ->
 // 150 (3 x 4; 2 x 8: 180), 48: 348 -> 285, 100: 558 -> 495, 200: 973 -> 927;
@@ -65,10 +70,12 @@ cudaError_t launch_decode_dm(const LaunchArgs& a, cudaStream_t st) {
   if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
   const int half = (a.M + 1) / 2;   // updates of a half-round
   auto fits = [&](int warps) { return smem_bytes_for<T, DM>(a.geo, a.M, warps) <= kMaxSmemBytes; };
-  auto resident = [&](int warps) {   // CTAs per network in one wave, 16 warps an SM
+  auto warps_per_sm = [&](int warps) {   // at most 16
     const long long per_sm = kSmemPerSm / (smem_bytes_for<T, DM>(a.geo, a.M, warps) + kSmemReservedPerCta);
-    return (per_sm * warps < 16 ? per_sm : 16 / warps) * sms / (4 * a.B);
+    return per_sm * warps < 16 ? per_sm * warps : 16;
   };
+  // CTAs per network in one wave.
+  auto resident = [&](int warps) { return warps_per_sm(warps) / warps * sms / (4 * a.B); };
   auto cluster = [&](int warps, long long n) {
     const long long cap = (half + warps - 1) / warps;
     n = n < cap ? n : cap;
@@ -76,12 +83,24 @@ cudaError_t launch_decode_dm(const LaunchArgs& a, cudaStream_t st) {
   };
   const bool small = half < 16;
   bool four = !fits(8) || small;
-  if (sizeof(T) == 8 && !four) four = resident(4) >= 3 && !(64 * a.B <= sms && half > 4 * kMaxCluster);
+  int least = 2, most = kMaxCluster;   // CTAs per network, before the cap of a warp per update
+  if (sizeof(T) == 8) {
+    if (!four) four = resident(4) >= 3 && !(64 * a.B <= sms && half > 4 * kMaxCluster);
+    if (small) least = kMaxCluster;
+  } else if (small) {
+    least = 1;
+  } else if (a.geo.k == 1 && resident(8) < 2) {
+    least = most = 1;
+    if (!four) four = resident(4) < 2 && warps_per_sm(4) >= warps_per_sm(8);
+  }
   const int warps = four ? 4 : 8;
   const long long n = resident(warps);
-  int cs = cluster(warps, small ? kMaxCluster : n < 2 ? 2 : n);
+  int cs = cluster(warps, n < least ? least : n > most ? most : n);
   if (4 * a.B * cs > 0x7fffffff) cs = 1;   // grid limit
-  return four ? launch_decode_nw<T, DM, 4>(a, cs, st) : launch_decode_nw<T, DM, 8>(a, cs, st);
+  if constexpr (sizeof(T) == 4) {
+    if (cs == 1) return four ? launch_decode_nw<T, DM, 4, false>(a, 1, st) : launch_decode_nw<T, DM, 8, false>(a, 1, st);
+  }
+  return four ? launch_decode_nw<T, DM, 4, true>(a, cs, st) : launch_decode_nw<T, DM, 8, true>(a, cs, st);
 }
 
 // D <= 4 in FP64 takes an instance of that capacity: 7 KB a warp instead of

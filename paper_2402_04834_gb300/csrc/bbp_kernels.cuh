@@ -1,13 +1,13 @@
 // Device code of the blockBP decoder (arXiv:2402.04834, Sec. III.D,
 // Algorithm 1, Remarks 2-8, Lemma 1) for sm_103a.
 //
-// One CTA, or a cluster of them in a small batch, decodes one (syndrome,
-// coset) pair from start to end: it builds the coset frame f_s * L (Algorithm
-// 1, first steps), keeps the MPS messages of all M directed block edges in a
-// global-memory arena, runs the chessboard schedule (Remark 8) with one warp
-// per message update and a barrier of the cluster between half-rounds,
-// evaluates Delta (Remark 4) and the Bethe read-out of Lemma 1.  No CTA ever
-// waits on one outside its cluster.
+// A cluster of CTAs, or one CTA by itself (launch_decode_dm has the rule),
+// decodes one (syndrome, coset) pair from start to end: it builds the coset
+// frame f_s * L (Algorithm 1, first steps), keeps the MPS messages of all M
+// directed block edges in a global-memory arena, runs the chessboard schedule
+// (Remark 8) with one warp per message update and a barrier of the cluster
+// between half-rounds, evaluates Delta (Remark 4) and the Bethe read-out of
+// Lemma 1.  No CTA ever waits on one outside its cluster.
 //
 // A warp owns a shared-memory workspace holding the running boundary MPS of
 // one block contraction.  The linear algebra is warp-cooperative on that
@@ -71,8 +71,10 @@ __device__ __forceinline__ P* cluster_peer(P* p, int rank) {
   asm("mapa.u64 %0, %1, %2;" : "=l"(q) : "l"((unsigned long long)p), "r"(rank));
   return reinterpret_cast<P*>(q);
 }
+template <bool CL>   // false: a CTA by itself, whose own barrier is enough
 __device__ __forceinline__ void cluster_barrier() {
-  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+  if constexpr (!CL) __syncthreads();
+  else asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
 }
 
 template <typename T> struct Eps;
@@ -191,7 +193,6 @@ struct Ctx {
   T* arena;                // this CTA's message arena
   const T* e0;             // the trivial border site (1, 0)
   int* cta_flags;       // rank 0's, when a cluster of CTAs shares the network
-  int cluster;          // CTAs that share the network
 };
 
 // ---------------------------------------------------------------------------
@@ -1192,7 +1193,7 @@ __device__ __noinline__ void damp(WarpWS<T, K, DM>& ws, const Ctx<T, K>& c, int 
 }
 
 // Store psi as message idx (bond dims checked against the slot bounds).
-template <typename T, int K, int DM>
+template <bool CL, typename T, int K, int DM>
 __device__ __noinline__ void store_msg(WarpWS<T, K, DM>& ws, const Ctx<T, K>& c, int idx, int w, int lane) {
   bool fits = true;
   for (int s = 0; s < w; ++s)
@@ -1204,20 +1205,23 @@ __device__ __noinline__ void store_msg(WarpWS<T, K, DM>& ws, const Ctx<T, K>& c,
   T* base = c.arena + c.msg_off[idx];
   for (int s = 0; s < w; ++s)
     warp_copy(base + msg_site_offset(s, w, c.D), ws.psi[s], ws.bond[s] * 2 * ws.bond[s + 1], lane);
-  for (int r = 0; r < c.cluster; ++r) {
-    int8_t* dm = cluster_peer(c.dims, r) + idx * (K + 1);
+  for (int r = 0; r < (CL ? cluster_size() : 1); ++r) {
+    int8_t* dm = (CL ? cluster_peer(c.dims, r) : c.dims) + idx * (K + 1);
     for (int s = lane; s <= w; s += 32) dm[s] = (int8_t)ws.bond[s];
   }
   __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
-// The decoder kernel: one cluster of CTAs per (syndrome, coset), a single CTA
-// where the batch fills the chip.  Messages are in the global arena; the tables
-// are built in every CTA, message bond dimensions and overlaps are written to
-// every CTA's copy, and the item counter, the flags and the read-out terms are
-// those of rank 0, so results do not depend on the cluster size.
-template <typename T, int K, int DM, int NW>
+// The decoder kernel: one cluster of CTAs per (syndrome, coset), of at least two
+// at any batch size but for short half-rounds and k = 1.  Messages are in the
+// global arena; the tables are built in every CTA, message bond dimensions and
+// overlaps are written to every CTA's copy, and the item counter, the flags and
+// the read-out terms are those of rank 0, so results do not depend on the
+// cluster size.
+// CL: may be launched as clusters; without, nothing of the above is compiled in
+// (an FP32 CTA by itself took up to 5 % longer through it, k = 1, d = 9).
+template <typename T, int K, int DM, int NW, bool CL>
 __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
   extern __shared__ __align__(16) unsigned char smem[];
   using WS = WarpWS<T, K, DM>;
@@ -1240,13 +1244,13 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
   WS* wsa = reinterpret_cast<WS*>(smem + Lo.ws);
 
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int CS = cluster_size(), cr = cluster_rank();
+  const int CS = CL ? cluster_size() : 1, cr = CL ? cluster_rank() : 0;
   const long long cta = blockIdx.x / CS;
   const long long shot = cta >> 2;
   const int coset = (int)(cta & 3);
   T* arena = a.arena + cta * (long long)a.arena_elems;
-  int* misc0 = cluster_peer(misc, 0);
-  double* rlog0 = cluster_peer(rlog, 0);
+  int* misc0 = CL ? cluster_peer(misc, 0) : misc;
+  double* rlog0 = CL ? cluster_peer(rlog, 0) : rlog;
 
   // Syndrome and the coset frame f_s * L (Algorithm 1; pure-error strings to
   // the right / bottom boundary, logicals on row 0 / column 0).
@@ -1296,7 +1300,6 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
   c.pI = a.pI_w; c.pE = a.pE_w;
   c.frame = frame; c.msg_of = msg_of; c.msg_off = msg_off; c.dims = dims;
   c.arena = arena; c.e0 = e0; c.cta_flags = &misc0[1];
-  c.cluster = CS;
 
   // Remark 2: uniform initial messages, bond 1, every site (1, 1)/sqrt(2).
   const T u = (T)0.70710678118654752440;
@@ -1310,7 +1313,13 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
     }
     for (int s = lane; s <= w; s += 32) dims[idx * (K + 1) + s] = 1;
   }
-  cluster_barrier();
+  cluster_barrier<CL>();
+
+  auto next_item = [&]() {
+    int item = 0;
+    if (lane == 0) item = atomicAdd(&misc0[0], 1);
+    return __shfl_sync(kFull, item, 0);
+  };
 
   WS& ws = wsa[warp];
   double delta = 0.0;
@@ -1320,9 +1329,7 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
       const int nwork = misc[2 + color];
       const int16_t* lst = work + color * M;
       for (;;) {
-        int item = 0;
-        if (lane == 0) item = atomicAdd(&misc0[0], 1);
-        item = __shfl_sync(kFull, item, 0);
+        const int item = next_item();
         if (item >= nwork) break;
         const int idx = lst[item];
         if (!dev_check(idx >= 0 && idx < M, &misc0[1])) continue;
@@ -1333,10 +1340,14 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
         damp(ws, c, idx, f.h, a.eta_w, lane);
         const double o = mps_overlap(ws, f.h, [&](int s) { return psi_site(ws, s); },
                                      [&](int s) { return msg_site(c, idx, f.h, s, false); }, lane);
-        store_msg(ws, c, idx, f.h, lane);
-        if (lane < CS) cluster_peer(ovl, lane)[idx] = o;
+        store_msg<CL>(ws, c, idx, f.h, lane);
+        if constexpr (CL) {
+          if (lane < CS) cluster_peer(ovl, lane)[idx] = o;
+        } else {
+          if (lane == 0) ovl[idx] = o;
+        }
       }
-      cluster_barrier();
+      cluster_barrier<CL>();
       if (tid == 0) misc[0] = 0;   // only rank 0's counts
       // Remark 4: Delta = sqrt(sum_i 2 - 2 <m_i^t | m_i^(t-1)>^2) / M.  Every
       // CTA sums its own copy of the overlaps between the two barriers: the
@@ -1349,7 +1360,7 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
         acc = warp_sum(acc);
         if (lane == 0) dsh[0] = sqrt(fmax(acc, 0.0)) / M;
       }
-      cluster_barrier();
+      cluster_barrier<CL>();
     }
     delta = dsh[0];
     it_done = it;
@@ -1366,13 +1377,11 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
     misc[4] = nedge;
     misc[0] = 0;
   }
-  cluster_barrier();
+  cluster_barrier<CL>();
   nedge = misc[4];
   const int nblk = nb * nb;
   for (;;) {
-    int item = 0;
-    if (lane == 0) item = atomicAdd(&misc0[0], 1);
-    item = __shfl_sync(kFull, item, 0);
+    const int item = next_item();
     if (item >= nblk + nedge) break;
     if (item < nblk) {
       const int I = item / nb, J = item % nb;
@@ -1403,7 +1412,7 @@ __global__ void __launch_bounds__(NW * 32) decode_kernel(KArgs<T> a) {
       }
     }
   }
-  cluster_barrier();
+  cluster_barrier<CL>();
   if (cr == 0 && warp == 0) {
     double acc = 0.0;
     for (int i = lane; i < nblk + nedge; i += 32) acc += rlog[i];

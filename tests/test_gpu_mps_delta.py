@@ -20,7 +20,7 @@ KEYS = ("logp", "delta", "iters", "flags", "decision")
 def test_early_exit_of_single_node_blocks(d, sizes):
     # M = 1088, 2400 and 3248 messages; with a rule of (warps, blocks per
     # network) by the batch these sizes run, on 152 SMs in FP64, as 8 x 8, 4 x 8,
-    # 4 x 5, 4 x 3 and 8 x 2, in FP32 as 8 x 8 down to 8 x 2 or 4 x 2.
+    # 4 x 5, 4 x 3 and 8 x 2, in FP32 as 8 x 8 down to 8 x 2 and without a cluster.
     p, n = 0.06, max(sizes)
     _, _, S = synth.sample_syndromes(8100 + d, 0, n, d, p)
     S = torch.from_numpy(S).cuda()
