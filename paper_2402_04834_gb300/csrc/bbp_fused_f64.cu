@@ -78,10 +78,13 @@ struct Shape {
   int lean = 0;   // > 0: every block update in register form, sized for this many CTAs per SM
 };
 
-// Compiled shapes in the order the default launch tries them: the
+// The shapes that can be asked for, in order of preference: the
 // register-form-only kernels where the geometry allows them, then
 // shared-memory messages where they leave room for the CTAs per SM of
-// target_blocks, then the same shape with its messages in the workspace.
+// target_blocks, then the same shape with its messages in the workspace.  They
+// decide what is accepted and the workspace it needs; a default launch takes its
+// kernel from fused_pick, and the first of these that fits where that has none
+// (k <= 3 and the geometries it leaves).
 constexpr Shape kShapesF32[] = {{8, 4, false, 4}, {8, 4, false, 3}, {8, 2, false, 4}, {8, 4, false}, {8, 4, true}, {8, 2, false},
                                 {8, 2, true}, {4, 2, false}, {4, 4, false}, {16, 1, false}, {8, 1, false},
                                 {4, 1, false}};

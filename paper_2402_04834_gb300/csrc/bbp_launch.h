@@ -12,8 +12,9 @@ namespace bbp {
 
 // Compile-time capacity of the instances: block side k <= kMaxK and bond
 // dimension D <= kMaxD; kWarps warps (message updates in flight) of the
-// smallest CTA, which decides what is accepted; kMaxCluster CTAs per network
-// (the portable cluster size).
+// smallest CTA of the MPS form, which runs where its shared memory fits (FP64
+// at D <= 4 needs less of it and reaches larger d); kMaxCluster CTAs per
+// network (the portable cluster size).
 constexpr int kMaxK = 4;
 constexpr int kMaxD = 8;
 constexpr int kWarps = 4;
