@@ -940,10 +940,26 @@ template <typename T, int NW, int G, int K, int LB = 0> struct FusedMinBlocks {
 
 // Position lists of a CTA: each colour's messages grouped by class, the
 // register forms first (class 2 shape + srev, so that a pass rarely mixes
-// both orders of the side messages), the node-by-node path last.
+// both orders of the side messages), the node-by-node path last; within a
+// class in any order, but in that of the blocks where every message is updated
+// node by node (k <= 3: neighbouring blocks share what L1 holds, and the short
+// updates of the edge blocks come last).
 constexpr int kClassNone = 2 * kShapes;
 constexpr int kClasses = kClassNone + 2;    // per colour: shapes x 2 orders, then none (R and D, L and U)
 template <int V> struct IntC { static constexpr int value = V; };
+
+// Messages of block (I, J)'s colour before its own in (I, J, dir) order.  A row's
+// blocks of one parity of J have two horizontal sides each, less one at either
+// end of the row.
+__device__ __forceinline__ int colour_rank(int nb, int I, int J) {
+  int n = 0;
+  for (int i = 0; i <= I; ++i) {
+    const int q = (I + J + i) & 1, end = i < I ? nb : J;               // blocks j < end, j = q mod 2
+    const int cnt = (end + 1 - q) >> 1, vertical = (i + 1 < nb) + (i > 0);
+    n += cnt * (2 + vertical) - (q == 0 && end > 0) - (end == nb && ((nb - 1) & 1) == q);
+  }
+  return n;
+}
 
 // Cosets c0 .. c0 + G - 1 of one syndrome decoded by the whole CTA: syn_src
 // holds the syndrome's m bytes and outputs go to row syn * 4 + coset.
@@ -1040,7 +1056,11 @@ __device__ __forceinline__ void fused_item(const KArgs<T>& a, const Geo g, const
       const int idx = message_index(nb, I, J, dir);
       if (dev_check(idx >= 0 && idx < M, &misc[4])) {
         meta[idx] = (int16_t)key;
-        rank[idx] = (int16_t)atomicAdd(&cls_n[class_of(I, J, dir)], 1);
+        int r = atomicAdd(&cls_n[class_of(I, J, dir)], 1);
+        if constexpr (K == 4 && !kLean) {
+          if (!reg) r = colour_rank(nb, I, J) + idx - message_index(nb, I, J, kDirR);
+        }
+        rank[idx] = (int16_t)r;
       }
       if constexpr (!kLean || kEven) msg_of[key] = (int16_t)idx;
     } else {
