@@ -56,7 +56,10 @@ cudaError_t launch_decode_nw(const LaunchArgs& a, int cluster, cudaStream_t st) 
 //   Half-rounds of fewer than 16 updates, whose warps the edge blocks leave
 //   idle, and k = 1, where an update is shorter than what a cluster adds to it,
 //   are shared only as far as CTAs are resident (d = 5, 150 syndromes: 1 x 4 9.4
-//   ms, 3 x 4 11.9; k = 1, d = 9, 76 syndromes: 1 x 8 7.7 ms, 2 x 8 8.8).
+//   ms, 3 x 4 11.9; k = 1, d = 9, 76 syndromes: 1 x 8 7.7 ms, 2 x 8 8.8).  A
+//   long half-round at k = 1 in a batch that fills the chip with four-warp CTAs
+//   takes those (d = 5, 144 updates, 300 syndromes: 1 x 4 7.4 ms, 1 x 8 8.5; d =
+//   3, 40 updates: 2.3 and 2.0).
 // ms, one CTA per network -> clusters: FP64 d = 11, 1 syndrome 223 -> 40 (8 x 8
 // warps; 8 x 4: 49), 5: 223 -> 59 (8 x 4; 8 x 8: 63), 12: 224 -> 84, 24: 225 ->
 // 150 (3 x 4; 2 x 8: 180), 48: 348 -> 285, 100: 558 -> 495, 200: 973 -> 927;
@@ -91,7 +94,7 @@ cudaError_t launch_decode_dm(const LaunchArgs& a, cudaStream_t st) {
     least = 1;
   } else if (a.geo.k == 1 && resident(8) < 2) {
     least = most = 1;
-    if (!four) four = resident(4) < 2 && warps_per_sm(4) >= warps_per_sm(8);
+    if (!four) four = half >= 64 && resident(4) < 2 && warps_per_sm(4) >= warps_per_sm(8);
   }
   const int warps = four ? 4 : 8;
   const long long n = resident(warps);
